@@ -289,7 +289,7 @@ int del_get_traffic(const del_ctx *ctx, int64_t *h2d_bytes, int64_t *d2h_bytes);
  * layers the selection can pick (e_min..e_max) and the last one; shadow tokens, counts and statistics of the other
  * layers are then not maintained, bit 8: the mma.sync flash-style prefill attention also where the tcgen05 one
  * (head dimension 128) would run, bit 9: the decode attention kernel does not request the O-projection's weights into
- * L2).  Returns the previous flags. */
+ * L2, bit 10: the layer GEMMs of every pass in the tcgen05 form that passes with many rows take, bit 11: of none).  Returns the previous flags. */
 int del_set_flags(del_ctx *ctx, int flags);
 
 /* With flag bit 3 set, per kernel class (0 QKV, 1 attention, 2 O-proj, 3 gate/up, 4 down, 5 draft LM

@@ -16,7 +16,7 @@ namespace {
 constexpr int PLAN_RING = 192;
 constexpr int CTR_RING = 4096;
 constexpr int FLAG_PDL = 1, FLAG_GRAPH = 2, FLAG_TC = 4, FLAG_TIMING = 8, FLAG_ONECTA = 16, FLAG_NO_BULK_PREFILL = 32,
-              FLAG_DECODE_ATTN_PREFILL = 64, FLAG_TRIM_ROWS = 128, FLAG_MMA_SYNC_PREFILL_ATTN = 256, FLAG_NO_WEIGHT_PREFETCH = 512;
+              FLAG_DECODE_ATTN_PREFILL = 64, FLAG_TRIM_ROWS = 128, FLAG_MMA_SYNC_PREFILL_ATTN = 256, FLAG_NO_WEIGHT_PREFETCH = 512, FLAG_TC_ROWS_ALL = 1024, FLAG_NO_TC_ROWS = 2048;
 enum { CLS_QKV = 0, CLS_ATTN, CLS_OPROJ, CLS_GATEUP, CLS_DOWN, CLS_LMHEAD, CLS_LMSTACK, CLS_OTHER, CLS_N };
 
 struct SeqHost {
@@ -77,6 +77,12 @@ struct del_ctx {
     TMap pf_xsl, pf_attl, pf_xml, pf_actl;                // ... and low parts
     TMap pf_q, pf_ql, kv_k, kv_v;                         // tcgen05 prefill attention: query buffers, paged cache
     bool pfa_ok = false;
+    // layer GEMMs of passes with many rows (rowgemm_tc.cu): tensor maps of inputs and weights, partial sums, tickets
+    TMap wt_xs, wt_xsl, wt_xd, wt_xdl, wt_att, wt_attl, wt_xm, wt_xml, wt_act, wt_actl;
+    std::vector<TMap> wt_q, wt_k, wt_v, wt_o, wt_g, wt_u, wt_d;
+    WtBuffers wt = {};
+    bool wt_ok = false;
+    int wt_rows_min = DEL_ROWS_MAX + 1;                   // rows from which on a pass takes that form
     std::vector<TMap> pf_wq, pf_wk, pf_wv, pf_wo, pf_wg, pf_wu, pf_wd;
     bool pf_ok = false;
     // mailbox of the draft loop's confidence check: pinned host memory that the finalise kernel writes directly
@@ -105,7 +111,7 @@ struct del_ctx {
 namespace {
 
 size_t carve_all(const del_shape &s, void *base, Dims &D, Buffers &B, int &R_max, int &n_vtiles,
-                 del_round_out **out_dev, float **dbg_dev, PfArgs *pf) {
+                 del_round_out **out_dev, float **dbg_dev, PfArgs *pf, WtBuffers *wt) {
     D.L = s.n_layers; D.d = s.d_model; D.nh = s.n_heads; D.nkv = s.n_kv_heads; D.hd = s.head_dim; D.F = s.d_ffn; D.V = s.vocab;
     D.B = s.max_batch;
     // slots of the hidden stack per sequence: what a round needs (g_max + 1 rows, the prefill window), raised to
@@ -183,6 +189,13 @@ size_t carve_all(const del_shape &s, void *base, Dims &D, Buffers &B, int &R_max
     pfa.ACT = c.take<bf16>(base, (size_t)PF_ROWS * D.F);
     pfa.ACTL = c.take<bf16>(base, (size_t)PF_ROWS * D.F);
     if (pf) *pf = pfa;
+    WtBuffers wtb;
+    wtb.n_tickets = std::max({rowgemm_tc_tiles(EPI_QKV, D), rowgemm_tc_tiles(EPI_GATEUP, D), rowgemm_tc_tiles(EPI_DOWN, D)});
+    wtb.xd = c.take<bf16>(base, (size_t)DEL_ROWS_MAX * D.d);
+    wtb.xdl = c.take<bf16>(base, (size_t)DEL_ROWS_MAX * D.d);
+    wtb.part = c.take<float>(base, (size_t)DEL_WT_CTAS * 2 * DEL_ROWS_MAX * 128);
+    wtb.ticket = c.take<int32_t>(base, (size_t)wtb.n_tickets);
+    if (wt) *wt = wtb;
     return (c.off + 255) & ~(size_t)255;
 }
 
@@ -367,6 +380,19 @@ CtlArgs ctl_base(const del_ctx *c, int plan_idx) {
     return a;
 }
 
+// Rows from which on a pass's layer GEMMs run on tcgen05 (rowgemm_tc.cu) rather than register streaming (rowgemm.cu).  The
+// former has a fixed cost of about 14 us per layer (four launches with a ticket and a merge at their end), the latter one
+// that grows with the rows and the weight bytes.  Measured, us per layer, register streaming / tcgen05:
+//   13B shape (635 MB)   5 rows 139 / 128,   8: 148 / 130,   13: 209 / 135
+//   8B shape (436 MB)    5 rows 104 / 107,   8: 107 / 107,    9: 138 / 110,   16: 155 / 114,   32: 268 / 140
+//   7B shape (405 MB)    5 rows  90 /  95,   8:  95 /  96,    9: 123 /  97,   16: 140 / 100,   32: 251 / 121
+//   1B shape (122 MB)    8 rows  50 /  63,   9:  65 /  67,   16:  74 /  68,   32: 112 /  92
+//   tiny (1.6 MB)        8 rows  18 /  34,  16:  24 /  34,   32:  33 /  47
+int rows_min_tc(const Dims &D) {
+    const double mb = 2e-6 * ((double)D.d * (D.nh + 2 * D.nkv) * D.hd + (double)D.nh * D.hd * D.d + 3.0 * D.d * D.F);
+    return mb >= 500 ? 5 : (mb >= 100 ? 9 : (mb >= 64 ? 17 : DEL_ROWS_MAX + 1));
+}
+
 struct PassInfo {
     int plan_idx, m, n_seg, max_rows, max_kv;
 };
@@ -382,15 +408,23 @@ PassInfo pass_info(const del_ctx *c, int plan_idx) {
 }
 
 // one decoder layer over the rows of a pass
-int run_layer(del_ctx *c, const PassInfo &pi, int l, bool write_exit) {
+int run_layer(del_ctx *c, const PassInfo &pi, int l, bool write_exit, bool first) {
     const Dims &D = c->D;
     const bool P = pdl(c);
+    // the layer before left its output by row of this pass as well
+    const bool dense = !first;
+    const bool wt = c->wt_ok && !(c->flags & FLAG_NO_TC_ROWS) && (pi.m >= c->wt_rows_min || (c->flags & FLAG_TC_ROWS_ALL));
     {
         GemmArgs a = gemm_base(c, pi.plan_idx, l);
         a.K = D.d;
         a.n_items = (D.nh + 2 * D.nkv) * (D.hd / 16);
         a.X = c->B.XS; a.XL = c->B.XSL;
         a.W0 = c->wq[l - 1]; a.W1 = c->wk[l - 1]; a.W2 = c->wv[l - 1];
+        if (wt && (dense || rowgemm_tc_fits(a))) {
+            TAG(CLS_QKV, 2.0 * (D.nh + 2 * D.nkv) * D.hd * D.d);
+            LAUNCH(launch_rowgemm_tc(EPI_QKV, a, c->wt_q[l - 1].b, c->wt_k[l - 1].b, c->wt_v[l - 1].b, dense ? c->wt_xd.b : c->wt_xs.b,
+                                     dense ? c->wt_xdl.b : c->wt_xsl.b, dense, c->wt, c->n_sms, c->st, P));
+        } else
         for (a.row0 = 0; a.row0 < pi.m; a.row0 += DEL_GEMM_ROWS) {
             if (a.row0) a.tile_ctr = next_counter(c);
             TAG(CLS_QKV, 2.0 * (D.nh + 2 * D.nkv) * D.hd * D.d);
@@ -434,6 +468,10 @@ int run_layer(del_ctx *c, const PassInfo &pi, int l, bool write_exit) {
         a.X = c->B.ATT; a.XL = c->B.ATTL;
         a.W0 = c->wo[l - 1];
         a.gain_a = c->ffn_norm[l - 1];
+        if (wt) {
+            TAG(CLS_OPROJ, 2.0 * D.d * D.nh * D.hd);
+            LAUNCH(launch_rowgemm_tc(EPI_OPROJ, a, c->wt_o[l - 1].b, nullptr, nullptr, c->wt_att.b, c->wt_attl.b, true, c->wt, c->n_sms, c->st, P));
+        } else
         for (a.row0 = 0; a.row0 < pi.m; a.row0 += DEL_GEMM_ROWS) {
             if (a.row0) a.tile_ctr = next_counter(c);
             TAG(CLS_OPROJ, 2.0 * D.d * D.nh * D.hd);
@@ -446,6 +484,10 @@ int run_layer(del_ctx *c, const PassInfo &pi, int l, bool write_exit) {
         a.n_items = D.F / 8;
         a.X = c->B.XM; a.XL = c->B.XML;
         a.W0 = c->w_gate[l - 1]; a.W1 = c->w_up[l - 1];
+        if (wt) {
+            TAG(CLS_GATEUP, 4.0 * D.F * D.d);
+            LAUNCH(launch_rowgemm_tc(EPI_GATEUP, a, c->wt_g[l - 1].b, c->wt_u[l - 1].b, nullptr, c->wt_xm.b, c->wt_xml.b, true, c->wt, c->n_sms, c->st, P));
+        } else
         for (a.row0 = 0; a.row0 < pi.m; a.row0 += DEL_GEMM_ROWS) {
             if (a.row0) a.tile_ctr = next_counter(c);
             TAG(CLS_GATEUP, 4.0 * D.F * D.d);
@@ -460,6 +502,10 @@ int run_layer(del_ctx *c, const PassInfo &pi, int l, bool write_exit) {
         a.W0 = c->w_down[l - 1];
         a.gain_a = l < D.L ? c->attn_norm[l] : nullptr;
         a.gain_b = write_exit ? c->final_norm : nullptr;
+        if (wt) {
+            TAG(CLS_DOWN, 2.0 * D.d * D.F);
+            LAUNCH(launch_rowgemm_tc(EPI_DOWN, a, c->wt_d[l - 1].b, nullptr, nullptr, c->wt_act.b, c->wt_actl.b, true, c->wt, c->n_sms, c->st, P));
+        } else
         for (a.row0 = 0; a.row0 < pi.m; a.row0 += DEL_GEMM_ROWS) {
             if (a.row0) a.tile_ctr = next_counter(c);
             TAG(CLS_DOWN, 2.0 * D.d * D.F);
@@ -536,8 +582,8 @@ int launch_draft_step(del_ctx *c, const DraftStep &st, const std::vector<int> &E
     for (size_t e = 0; e < Es.size(); ++e) {
         if (st.sub_idx[e] < 0) break;
         const PassInfo pi = pass_info(c, st.sub_idx[e]);
-        for (; l <= Es[e]; ++l) {
-            int rc = run_layer(c, pi, l, l == Es[e]);
+        for (const int l0 = l; l <= Es[e]; ++l) {
+            int rc = run_layer(c, pi, l, l == Es[e], l == l0);
             if (rc) return rc;
         }
     }
@@ -787,8 +833,8 @@ int enqueue_verify(del_ctx *c, const std::vector<Job> &jobs) {
         const int l_last = k < Es.size() ? Es[k] : c->D.L;
         if (idx[k] < 0) { l = l_last + 1; continue; }
         const PassInfo pi = pass_info(c, idx[k]);
-        for (; l <= l_last; ++l) {
-            rc = run_layer(c, pi, l, false);
+        for (const int l0 = l; l <= l_last; ++l) {
+            rc = run_layer(c, pi, l, false, l == l0);
             if (rc) return rc;
         }
     }
@@ -953,6 +999,7 @@ int read_out(del_ctx *c) {
         // a bounded device-side wait expired; clear the word so that the context stays usable
         snprintf(c->err, sizeof(c->err), "device wait expired (code %d)", *err_host);
         cudaMemsetAsync(c->B.ERR, 0, sizeof(int32_t), c->st);
+        cudaMemsetAsync(c->wt.ticket, 0, sizeof(int32_t) * c->wt.n_tickets, c->st);      // a launch that gave up leaves arrivals behind
         return DEL_ETIMEOUT;
     }
     return DEL_OK;
@@ -993,7 +1040,7 @@ extern "C" {
 size_t del_workspace_bytes(const del_shape *shape) {
     if (validate(shape) != DEL_OK) return 0;
     Dims D; Buffers B; int R, nv; del_round_out *o; float *dbg;
-    return carve_all(*shape, nullptr, D, B, R, nv, &o, &dbg, nullptr);
+    return carve_all(*shape, nullptr, D, B, R, nv, &o, &dbg, nullptr, nullptr);
 }
 
 int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const del_kv *kv, void *workspace,
@@ -1009,7 +1056,7 @@ int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const 
     del_ctx *c = new (std::nothrow) del_ctx();
     if (!c) return DEL_ENOSPC;
     c->sh = *shape;
-    carve_all(*shape, workspace, c->D, c->B, c->R_max, c->n_vtiles, &c->out_dev, &c->dbg_dev, &c->pf);
+    carve_all(*shape, workspace, c->D, c->B, c->R_max, c->n_vtiles, &c->out_dev, &c->dbg_dev, &c->pf, &c->wt);
     c->B.KP = (bf16 *)kv->k_pages; c->B.VP = (bf16 *)kv->v_pages; c->B.PT = kv->page_table;
     c->B.rope_cos = w->rope_cos; c->B.rope_sin = w->rope_sin;
     c->tok_emb = (const bf16 *)w->tok_emb; c->final_norm = (const bf16 *)w->final_norm; c->lm_head = (const bf16 *)w->lm_head;
@@ -1095,6 +1142,25 @@ int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const 
         maps(c->pf_wd, c->w_down, d, F, bn_narrow);
         c->pf.bn_narrow = (int32_t)bn_narrow;
         c->pf_ok = ok;
+        maps(c->wt_q, c->wq, qd, d, 128);
+        maps(c->wt_k, c->wk, kvd, d, 128);
+        maps(c->wt_v, c->wv, kvd, d, 128);
+        maps(c->wt_o, c->wo, d, qd, 128);
+        maps(c->wt_g, c->w_gate, F, d, 64);
+        maps(c->wt_u, c->w_up, F, d, 64);
+        maps(c->wt_d, c->w_down, d, F, 128);
+        const uint64_t stack_rows = ((uint64_t)L + 1) * c->D.B * c->D.S;
+        c->wt_rows_min = rows_min_tc(c->D);
+        c->wt_ok = ok && rowgemm_tc_supported(c->D) && lmhead_tc_make_map(c->wt_xs.b, c->B.XS, stack_rows, d, 8) == 0 &&
+                   lmhead_tc_make_map(c->wt_xsl.b, c->B.XSL, stack_rows, d, 8) == 0 &&
+                   lmhead_tc_make_map(c->wt_xd.b, c->wt.xd, DEL_ROWS_MAX, d, 16) == 0 &&
+                   lmhead_tc_make_map(c->wt_xdl.b, c->wt.xdl, DEL_ROWS_MAX, d, 16) == 0 &&
+                   lmhead_tc_make_map(c->wt_att.b, c->B.ATT, DEL_ROWS_MAX, qd, 16) == 0 &&
+                   lmhead_tc_make_map(c->wt_attl.b, c->B.ATTL, DEL_ROWS_MAX, qd, 16) == 0 &&
+                   lmhead_tc_make_map(c->wt_xm.b, c->B.XM, DEL_ROWS_MAX, d, 16) == 0 &&
+                   lmhead_tc_make_map(c->wt_xml.b, c->B.XML, DEL_ROWS_MAX, d, 16) == 0 &&
+                   lmhead_tc_make_map(c->wt_act.b, c->B.ACT, DEL_ROWS_MAX, F, 16) == 0 &&
+                   lmhead_tc_make_map(c->wt_actl.b, c->B.ACTL, DEL_ROWS_MAX, F, 16) == 0;
         c->pfa_ok = ok && prefill_attention_tc_supported(c->D) &&
                     lmhead_tc_make_map(c->pf_q.b, c->pf.Q, PF_ROWS, qd, 128) == 0 &&
                     lmhead_tc_make_map(c->pf_ql.b, c->pf.QL, PF_ROWS, qd, 128) == 0 &&
@@ -1170,7 +1236,7 @@ int del_prefill(del_ctx *c, int sq, const int32_t *prompt, int n_prompt, int max
         LAUNCH(launch_embed(ca, ch.second, c->st, pdl(c)));
         const PassInfo pi = pass_info(c, idx);
         for (int l = 1; l <= c->D.L; ++l) {
-            rc = run_layer(c, pi, l, false);
+            rc = run_layer(c, pi, l, false, l == 1);
             if (rc) return rc;
         }
     }

@@ -45,6 +45,20 @@ cudaError_t launch_rowgemm(int epi, const GemmArgs &a, int m, int n_sms, cudaStr
 // CTAs an LM-head launch of m rows uses (= number of arg-max partials it leaves per row)
 int rowgemm_lmhead_grid(int n_items, int m, int n_sms, int ctas_per_sm);
 
+// The layer GEMMs of passes with many rows on tcgen05 (rowgemm_tc.cu): all rows of the pass in one launch
+#define DEL_WT_CTAS 160        // most CTAs of such a launch (partial sums in the workspace: 2 x 128 x 64 floats each)
+struct WtBuffers {
+    bf16 *xd, *xdl;            // [ROWS][d] the next layer's input by row of the pass, written by DOWN beside the hidden stack
+    float *part;               // partial sums of tiles that several CTAs share
+    int32_t *ticket;           // [tiles] arrivals at such a tile; zero between launches
+    int32_t n_tickets;
+};
+int rowgemm_tc_tiles(int epi, const Dims &D);
+bool rowgemm_tc_supported(const Dims &D);
+bool rowgemm_tc_fits(const GemmArgs &a);               // whether a QKV launch can read the pass's rows from the hidden stack
+cudaError_t launch_rowgemm_tc(int epi, const GemmArgs &a, const void *map_w0, const void *map_w1, const void *map_w2, const void *map_x,
+                              const void *map_xl, bool dense, const WtBuffers &b, int n_sms, cudaStream_t st, bool pdl);
+
 struct AttnArgs {
     Dims D;
     Buffers B;

@@ -1,0 +1,59 @@
+"""Layer passes with many rows: the tcgen05 form of the layer GEMMs against the register-streaming form and the oracle."""
+import numpy as np
+import pytest
+
+import synth
+from cases import TINY, TINY_GQA
+from parity import ref_from_oracle, run_batch
+
+pytestmark = pytest.mark.gpu
+
+# widths that end inside a tile (128 rows), a K block (128) and a partial sum's group; one kv head of 64 features
+RAGGED = synth.small_variant(TINY, name="ragged", d_model=288, n_heads=5, n_kv_heads=1, head_dim=64, d_ffn=272, emb_scale=10.0,
+                             gain_spread=0.1, init_window=32, seed=31)
+HD128 = synth.small_variant(TINY, name="hd128", d_model=512, n_heads=6, n_kv_heads=3, head_dim=128, d_ffn=1040, emb_scale=10.0,
+                            gain_spread=0.1, init_window=32, seed=32)
+
+
+def make_ctx(cfg, w, **kw):
+    import paper_2504_05598_b200 as dl
+    return dl.DelContext(dl.make_shape(cfg, **kw), dl.upload_weights(w))
+
+
+@pytest.mark.parametrize("cfg", [RAGGED, HD128], ids=lambda c: c.name)
+@pytest.mark.parametrize("rows", [1, 8, 9, 16, 17, 32, 33, 48, 49, 64])
+def test_forms_agree_on_one_pass(cfg, rows):
+    """A prompt of rows + 1 positions is a pass of `rows` rows and a window of 1 row (init_window 1): the cache rows the
+    first writes and the hidden states of the second, with both forms.  The two differ in the order of fp32 sums and so in
+    single roundings of the bf16 cache (2^-9 of a value each, of random sign) and of the 16-bit activation pairs: 2^-8 of a
+    vector's norm bounds both."""
+    import paper_2504_05598_b200 as dl
+    cfg = synth.small_variant(cfg, init_window=1, prompt_len=rows + 1, gen_len=4)
+    w = synth.make_weights(cfg)
+    ctx = make_ctx(cfg, w)
+    got = {}
+    for form in (dl.FLAG_NO_TC_ROWS, dl.FLAG_TC_ROWS_ALL):
+        ctx.set_flags(dl.FLAG_PDL | dl.FLAG_TC | dl.FLAG_NO_BULK_PREFILL | form)
+        ctx.prefill(0, synth.make_prompt(cfg), 2)
+        got[form] = ([ctx.get_hidden(0, l, 0) for l in range(1, cfg.n_layers + 1)] +
+                     [x for l in range(1, cfg.n_layers + 1) for pos in range(rows + 1) for x in ctx.get_kv(0, l, pos)])
+    for a, b in zip(*got.values()):
+        assert np.linalg.norm(a - b) <= 2.0 ** -8 * np.linalg.norm(a)
+    ctx.close()
+
+
+@pytest.mark.parametrize("batch,g_max", [(1, 12), (3, 9), (7, 8), (8, 7), (16, 3)])
+def test_rounds_against_oracle(batch, g_max):
+    """Whole rounds with every pass in the tcgen05 form: several sequences, whose rows the first layer of a pass gathers
+    from the hidden stack in groups of eight ((16, 3): more groups than fit, that launch streams through registers)."""
+    import paper_2504_05598_b200 as dl
+    cfg = synth.small_variant(TINY_GQA, batch=batch, g_max=g_max, prompt_len=40, gen_len=20)
+    w = synth.make_weights(cfg)
+    ctx = make_ctx(cfg, w)
+    ctx.set_flags(dl.FLAG_PDL | dl.FLAG_TC | dl.FLAG_TC_ROWS_ALL)
+    refs = [ref_from_oracle(cfg, w, synth.make_prompt(cfg, s)) for s in range(batch)]
+    reps = run_batch(ctx, refs, cfg.gen_len)
+    for s, rep in enumerate(reps):
+        assert rep.ok(), (s, rep.failures[:5])
+        assert rep.rounds == len(refs[s].rounds)
+    ctx.close()
