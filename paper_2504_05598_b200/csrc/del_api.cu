@@ -79,11 +79,10 @@ struct del_ctx {
     bool pfa_ok = false;
     // layer GEMMs of passes with many rows (rowgemm_tc.cu): tensor maps of inputs and weights, partial sums, tickets
     TMap wt_xs, wt_xsl, wt_xd, wt_xdl, wt_att, wt_attl, wt_xm, wt_xml, wt_act, wt_actl;
-    std::vector<TMap> wt_q, wt_k, wt_v, wt_o, wt_g, wt_u, wt_d;
+    std::vector<TMap> wt_q, wt_k, wt_v, wt_o, wt_g, wt_u, wt_d;          // (also the prefill's)
     WtBuffers wt = {};
     bool wt_ok = false;
     int wt_rows_min = DEL_ROWS_MAX + 1;                   // rows from which on a pass takes that form
-    std::vector<TMap> pf_wq, pf_wk, pf_wv, pf_wo, pf_wg, pf_wu, pf_wd;
     bool pf_ok = false;
     // mailbox of the draft loop's confidence check: pinned host memory that the finalise kernel writes directly
     volatile float *post_conf = nullptr;
@@ -109,6 +108,9 @@ struct del_ctx {
 };
 
 namespace {
+
+// rows of the bulk prefill's chunk buffers: a chunk, or all a sequence can hold (whole 128-row tiles)
+int prefill_rows(const del_shape &s) { return std::min(PF_ROWS, (s.max_seq + 127) / 128 * 128); }
 
 size_t carve_all(const del_shape &s, void *base, Dims &D, Buffers &B, int &R_max, int &n_vtiles,
                  del_round_out **out_dev, float **dbg_dev, PfArgs *pf, WtBuffers *wt) {
@@ -172,25 +174,26 @@ size_t carve_all(const del_shape &s, void *base, Dims &D, Buffers &B, int &R_max
     B.ERR = c.take<int32_t>(base, 64);           // right behind the results: one copy brings both to the host
     *dbg_dev = c.take<float>(base, (size_t)std::max(D.V, 2 * D.nkv * D.hd));
     // chunk buffers of the bulk prefill (PF_ROWS prompt positions)
+    const int pf_rows = prefill_rows(s);
     PfArgs pfa;
     memset(&pfa, 0, sizeof(pfa));
     pfa.n_ssp = prefill_tc_nssp(D);
-    pfa.H = c.take<float>(base, (size_t)PF_ROWS * D.d);
-    pfa.XS = c.take<bf16>(base, (size_t)PF_ROWS * D.d);
-    pfa.XSL = c.take<bf16>(base, (size_t)PF_ROWS * D.d);
-    pfa.SSP = c.take<float>(base, (size_t)PF_ROWS * pfa.n_ssp);
-    pfa.Q = c.take<bf16>(base, (size_t)PF_ROWS * qd);
-    pfa.QL = c.take<bf16>(base, (size_t)PF_ROWS * qd);
-    pfa.ATT = c.take<bf16>(base, (size_t)PF_ROWS * qd);
-    pfa.ATTL = c.take<bf16>(base, (size_t)PF_ROWS * qd);
-    pfa.XM = c.take<bf16>(base, (size_t)PF_ROWS * D.d);
-    pfa.XML = c.take<bf16>(base, (size_t)PF_ROWS * D.d);
-    pfa.SSPM = c.take<float>(base, (size_t)PF_ROWS * pfa.n_ssp);
-    pfa.ACT = c.take<bf16>(base, (size_t)PF_ROWS * D.F);
-    pfa.ACTL = c.take<bf16>(base, (size_t)PF_ROWS * D.F);
+    pfa.H = c.take<float>(base, (size_t)pf_rows * D.d);
+    pfa.XS = c.take<bf16>(base, (size_t)pf_rows * D.d);
+    pfa.XSL = c.take<bf16>(base, (size_t)pf_rows * D.d);
+    pfa.SSP = c.take<float>(base, (size_t)pf_rows * pfa.n_ssp);
+    pfa.Q = c.take<bf16>(base, (size_t)pf_rows * qd);
+    pfa.QL = c.take<bf16>(base, (size_t)pf_rows * qd);
+    pfa.ATT = c.take<bf16>(base, (size_t)pf_rows * qd);
+    pfa.ATTL = c.take<bf16>(base, (size_t)pf_rows * qd);
+    pfa.XM = c.take<bf16>(base, (size_t)pf_rows * D.d);
+    pfa.XML = c.take<bf16>(base, (size_t)pf_rows * D.d);
+    pfa.SSPM = c.take<float>(base, (size_t)pf_rows * pfa.n_ssp);
+    pfa.ACT = c.take<bf16>(base, (size_t)pf_rows * D.F);
+    pfa.ACTL = c.take<bf16>(base, (size_t)pf_rows * D.F);
     if (pf) *pf = pfa;
     WtBuffers wtb;
-    wtb.n_tickets = std::max({rowgemm_tc_tiles(EPI_QKV, D), rowgemm_tc_tiles(EPI_GATEUP, D), rowgemm_tc_tiles(EPI_DOWN, D)});
+    wtb.n_tickets = std::max({DEL_WT_CTAS, rowgemm_tc_tiles(EPI_QKV, D), rowgemm_tc_tiles(EPI_GATEUP, D), rowgemm_tc_tiles(EPI_DOWN, D)});
     wtb.xd = c.take<bf16>(base, (size_t)DEL_ROWS_MAX * D.d);
     wtb.xdl = c.take<bf16>(base, (size_t)DEL_ROWS_MAX * D.d);
     wtb.part = c.take<float>(base, (size_t)DEL_WT_CTAS * 2 * DEL_ROWS_MAX * 128);
@@ -740,8 +743,7 @@ int prefill_bulk(del_ctx *c, int sq, int n_pos, int win0) {
         for (int l = 1; l <= D.L; ++l) {
             a.layer = l;
             a.K = D.d;
-            a.n_ntiles = prefill_tc_ntiles(PF_QKV, D);
-            LAUNCH(launch_prefill_gemm(PF_QKV, c->pf_xs.b, c->pf_xsl.b, c->pf_wq[l - 1].b, c->pf_wk[l - 1].b, c->pf_wv[l - 1].b, a, c->n_sms, c->st, P));
+            LAUNCH(launch_prefill_gemm(PF_QKV, c->pf_xs.b, c->pf_xsl.b, c->wt_q[l - 1].b, c->wt_k[l - 1].b, c->wt_v[l - 1].b, a, c->n_sms, c->st, P));
             if (l == D.L && !has_window) break;       // of the last layer only the keys and values are needed
             if (!(c->flags & FLAG_DECODE_ATTN_PREFILL)) {
                 // one flash-style pass over the chunk's rows and all keys up to each row's position
@@ -776,16 +778,13 @@ int prefill_bulk(del_ctx *c, int sq, int n_pos, int win0) {
                 LAUNCH(launch_attention(at, 1, c->st, P));
             }
             a.K = D.nh * D.hd;
-            a.n_ntiles = prefill_tc_ntiles(PF_OPROJ, D);
             a.gain = c->ffn_norm[l - 1];
-            LAUNCH(launch_prefill_gemm(PF_OPROJ, c->pf_att.b, c->pf_attl.b, c->pf_wo[l - 1].b, nullptr, nullptr, a, c->n_sms, c->st, P));
+            LAUNCH(launch_prefill_gemm(PF_OPROJ, c->pf_att.b, c->pf_attl.b, c->wt_o[l - 1].b, nullptr, nullptr, a, c->n_sms, c->st, P));
             a.K = D.d;
-            a.n_ntiles = prefill_tc_ntiles(PF_GATEUP, D);
-            LAUNCH(launch_prefill_gemm(PF_GATEUP, c->pf_xm.b, c->pf_xml.b, c->pf_wg[l - 1].b, c->pf_wu[l - 1].b, nullptr, a, c->n_sms, c->st, P));
+            LAUNCH(launch_prefill_gemm(PF_GATEUP, c->pf_xm.b, c->pf_xml.b, c->wt_g[l - 1].b, c->wt_u[l - 1].b, nullptr, a, c->n_sms, c->st, P));
             a.K = D.F;
-            a.n_ntiles = prefill_tc_ntiles(PF_DOWN, D);
             a.gain = l < D.L ? c->attn_norm[l] : nullptr;      // the next layer's attention norm
-            LAUNCH(launch_prefill_gemm(PF_DOWN, c->pf_act.b, c->pf_actl.b, c->pf_wd[l - 1].b, nullptr, nullptr, a, c->n_sms, c->st, P));
+            LAUNCH(launch_prefill_gemm(PF_DOWN, c->pf_act.b, c->pf_actl.b, c->wt_d[l - 1].b, nullptr, nullptr, a, c->n_sms, c->st, P));
         }
     }
     return DEL_OK;
@@ -1117,31 +1116,22 @@ int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const 
                lmhead_tc_make_map(c->map_x, c->B.XN, (uint64_t)c->R_max + 128, (uint64_t)shape->d_model, 128) == 0 &&
                lmhead_tc_make_map(c->map_w, c->lm_head, (uint64_t)shape->vocab, (uint64_t)shape->d_model, 256) == 0;
     {
-        // tensor maps of the bulk prefill: activations in boxes of 128 rows, weights of 256 (gate / up: 128)
+        // tensor maps of the bulk prefill and of the weights: boxes of 128 rows (gate / up: 64)
+        const uint64_t pf_rows = prefill_rows(*shape);
         const uint64_t d = shape->d_model, qd = (uint64_t)shape->n_heads * shape->head_dim,
                        kvd = (uint64_t)shape->n_kv_heads * shape->head_dim, F = shape->d_ffn;
-        bool ok = lmhead_tc_make_map(c->pf_xs.b, c->pf.XS, PF_ROWS, d, 128) == 0 &&
-                  lmhead_tc_make_map(c->pf_att.b, c->pf.ATT, PF_ROWS, qd, 128) == 0 &&
-                  lmhead_tc_make_map(c->pf_xm.b, c->pf.XM, PF_ROWS, d, 128) == 0 &&
-                  lmhead_tc_make_map(c->pf_act.b, c->pf.ACT, PF_ROWS, F, 128) == 0 &&
-                  lmhead_tc_make_map(c->pf_xsl.b, c->pf.XSL, PF_ROWS, d, 128) == 0 &&
-                  lmhead_tc_make_map(c->pf_attl.b, c->pf.ATTL, PF_ROWS, qd, 128) == 0 &&
-                  lmhead_tc_make_map(c->pf_xml.b, c->pf.XML, PF_ROWS, d, 128) == 0 &&
-                  lmhead_tc_make_map(c->pf_actl.b, c->pf.ACTL, PF_ROWS, F, 128) == 0;
+        bool ok = lmhead_tc_make_map(c->pf_xs.b, c->pf.XS, pf_rows, d, 128) == 0 &&
+                  lmhead_tc_make_map(c->pf_att.b, c->pf.ATT, pf_rows, qd, 128) == 0 &&
+                  lmhead_tc_make_map(c->pf_xm.b, c->pf.XM, pf_rows, d, 128) == 0 &&
+                  lmhead_tc_make_map(c->pf_act.b, c->pf.ACT, pf_rows, F, 128) == 0 &&
+                  lmhead_tc_make_map(c->pf_xsl.b, c->pf.XSL, pf_rows, d, 128) == 0 &&
+                  lmhead_tc_make_map(c->pf_attl.b, c->pf.ATTL, pf_rows, qd, 128) == 0 &&
+                  lmhead_tc_make_map(c->pf_xml.b, c->pf.XML, pf_rows, d, 128) == 0 &&
+                  lmhead_tc_make_map(c->pf_actl.b, c->pf.ACTL, pf_rows, F, 128) == 0;
         auto maps = [&](std::vector<del_ctx::TMap> &dst, const std::vector<const bf16 *> &w, uint64_t rows, uint64_t cols, uint32_t box) {
             dst.resize(L);
             for (int l = 0; l < L && ok; ++l) ok = lmhead_tc_make_map(dst[l].b, w[l], rows, cols, box) == 0;
         };
-        maps(c->pf_wq, c->wq, qd, d, 256);
-        maps(c->pf_wk, c->wk, kvd, d, 256);
-        maps(c->pf_wv, c->wv, kvd, d, 256);
-        const uint32_t bn_narrow = (uint32_t)prefill_tc_narrow(c->D);
-        maps(c->pf_wo, c->wo, d, qd, bn_narrow);
-        maps(c->pf_wg, c->w_gate, F, d, 128);
-        maps(c->pf_wu, c->w_up, F, d, 128);
-        maps(c->pf_wd, c->w_down, d, F, bn_narrow);
-        c->pf.bn_narrow = (int32_t)bn_narrow;
-        c->pf_ok = ok;
         maps(c->wt_q, c->wq, qd, d, 128);
         maps(c->wt_k, c->wk, kvd, d, 128);
         maps(c->wt_v, c->wv, kvd, d, 128);
@@ -1149,6 +1139,7 @@ int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const 
         maps(c->wt_g, c->w_gate, F, d, 64);
         maps(c->wt_u, c->w_up, F, d, 64);
         maps(c->wt_d, c->w_down, d, F, 128);
+        c->pf_ok = ok;
         const uint64_t stack_rows = ((uint64_t)L + 1) * c->D.B * c->D.S;
         c->wt_rows_min = rows_min_tc(c->D);
         c->wt_ok = ok && rowgemm_tc_supported(c->D) && lmhead_tc_make_map(c->wt_xs.b, c->B.XS, stack_rows, d, 8) == 0 &&
@@ -1162,10 +1153,12 @@ int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const 
                    lmhead_tc_make_map(c->wt_act.b, c->B.ACT, DEL_ROWS_MAX, F, 16) == 0 &&
                    lmhead_tc_make_map(c->wt_actl.b, c->B.ACTL, DEL_ROWS_MAX, F, 16) == 0;
         c->pfa_ok = ok && prefill_attention_tc_supported(c->D) &&
-                    lmhead_tc_make_map(c->pf_q.b, c->pf.Q, PF_ROWS, qd, 128) == 0 &&
-                    lmhead_tc_make_map(c->pf_ql.b, c->pf.QL, PF_ROWS, qd, 128) == 0 &&
+                    lmhead_tc_make_map(c->pf_q.b, c->pf.Q, pf_rows, qd, 128) == 0 &&
+                    lmhead_tc_make_map(c->pf_ql.b, c->pf.QL, pf_rows, qd, 128) == 0 &&
                     prefill_attention_tc_make_maps(c->kv_k.b, c->kv_v.b, c->B.KP, c->B.VP, c->D, shape->n_pages) == 0;
         c->pf.D = c->D;
+        c->pf.part = c->wt.part;
+        c->pf.ticket = c->wt.ticket;
         c->pf.KP = c->B.KP; c->pf.VP = c->B.VP; c->pf.PT = c->B.PT;
         c->pf.rope_cos = c->B.rope_cos; c->pf.rope_sin = c->B.rope_sin;
         c->pf.err = c->B.ERR;
@@ -1213,8 +1206,10 @@ int del_prefill(del_ctx *c, int sq, const int32_t *prompt, int n_prompt, int max
     // chunks of <= S positions; the last chunk is exactly the window so that its hidden states stay
     // in slots 0..W-1 of the stack
     std::vector<std::pair<int, int>> chunks;
-    // long prompts go through the tensor-core prefill as a whole; short ones through the decode kernels
-    if (c->pf_ok && !(c->flags & FLAG_NO_BULK_PREFILL) && n_prompt - W >= 64) {
+    // From 40 positions on a prompt goes through the tensor-core prefill as a whole; shorter ones take a pass or two of the
+    // decode kernels.  us per layer, decode kernels / prefill kernels: 7B shape 36 positions 225 / 222, 45: 247 / 223, 77: 286 /
+    // 229; 1B 36: 158 / 168, 40: 168 / 169, 45: 184 / 167, 77: 239 / 181; 13B 33: 307 / 255; tiny 40: 60 / 66, 48: 68 / 67.
+    if (c->pf_ok && !(c->flags & FLAG_NO_BULK_PREFILL) && n_prompt >= 40 && n_prompt - W >= 8) {
         rc = prefill_bulk(c, sq, n_prompt, n_prompt - W);
         if (rc) return rc;
     } else {

@@ -174,18 +174,23 @@ cudaError_t launch_lmhead_tc(const void *map_x, const void *map_w, float *part_v
                              int n_sms, cudaStream_t st, bool pdl);
 
 // Prompt prefill on tcgen05 (prefill_tc.cu): tiled GEMMs over up to PF_ROWS prompt positions of one sequence
-// with the layer's element-wise work fused into the epilogues.  All buffers hold PF_ROWS rows.
-#define PF_ROWS 512
+// with the layer's element-wise work fused into the epilogues.  All buffers hold PF_ROWS rows (fewer if max_seq is smaller).
+// 1024 rather than 512: twice the tiles leave less of the last wave of tiles idle (7B shape, 1000 positions: gate/up 5 waves
+// instead of 3 + 3, QKV 3 instead of 2 + 2; 860 -> 679 us per layer), while a chunk's activations (57 MB for the 13B
+// shape's down projection) still fit L2 beside the weights in flight.
+#define PF_ROWS 1024
 enum { PF_QKV = 0, PF_OPROJ = 1, PF_GATEUP = 2, PF_DOWN = 3 };
 struct PfArgs {
     Dims D;
     int32_t M, K;              // valid rows of the chunk, in-features of this GEMM
-    int32_t n_ntiles;          // output tiles of this GEMM (prefill_tc_ntiles)
-    int32_t n_ssp;             // partial sums of squares per row (= output tiles of a d-wide GEMM)
+    int32_t n_ntiles, bn, k_parts;     // set by the launch: output tiles, their width, parts of K per tile
+    float *part;               // [parts][tiles][128][bn] partial sums, [tiles] tickets (zero between launches)
+    int32_t *ticket;
+    int32_t n_ssp;             // partial sums of squares per row (one per 64 columns)
     int32_t layer, seq, pos0;  // 1-based layer; the rows are positions pos0 .. pos0 + M - 1 of sequence seq
     float *H;                  // [PF_ROWS][d] residual stream, updated in place
     bf16 *XS, *XSL;            // [PF_ROWS][d] h * attention-norm gain (high / low part): input of QKV, written by DOWN
-    float *SSP;                // [PF_ROWS][n_ssp] sums of squares of h per output tile of DOWN (QKV's 1/rms)
+    float *SSP;                // [PF_ROWS][n_ssp] partial sums of squares of h (QKV's 1/rms)
     bf16 *Q, *QL, *ATT, *ATTL; // [PF_ROWS][nh * hd] queries, attention output (each as high / low part)
     bf16 *XM, *XML;            // [PF_ROWS][d] h_mid * ffn-norm gain (high / low part), written by OPROJ
     float *SSPM;               // [PF_ROWS][n_ssp]
@@ -194,16 +199,14 @@ struct PfArgs {
     bf16 *KP, *VP;             // paged cache
     const int32_t *PT;
     const float *rope_cos, *rope_sin;
+    int32_t rope_vec, vp_vec;  // both tables / the value pages 16-byte aligned (set by the launch)
     int32_t *err;
     // rows at positions >= win0 belong to the window that seeds the acceptance statistics: their hidden state
     // after every layer is also stored in the hidden stack (slot = position - win0)
     float *stackH;
     int32_t win0;
-    int32_t bn_narrow;         // tile width of O-proj and down (prefill_tc_narrow)
 };
-int prefill_tc_ntiles(int epi, const Dims &D);
-int prefill_tc_narrow(const Dims &D);          // tile width of O-proj and down for this shape
-int prefill_tc_nssp(const Dims &D);            // partial sums of squares per row (one per 128 columns)
+int prefill_tc_nssp(const Dims &D);            // partial sums of squares per row
 
 // Causal attention of a prefill chunk (prefill_attn.cu): rows 0..M-1 of Q (positions pos0 + row of sequence seq)
 // against the paged cache of `layer` (which already holds the chunk's own keys and values) -> ATT.

@@ -16,12 +16,13 @@
 // two MMAs on the same weight tile, one per part, into the same accumulator, so that the prompt's keys, values
 // and hidden states carry the same accuracy as those the decode kernels make.
 //
-// CTA tile 128 rows x 256 output features (128 for the two d-wide projections, whose 256-wide tiles would
-// fill less than half of the SMs), K blocks of 64 (one 128-byte swizzle span), same roles as
-// the stacked LM head: warp 0 issues TMA loads into a 3-stage shared-memory ring, warp 1 issues
-// tcgen05.mma into one of two 256-column accumulators in tensor memory, warps 2-5 read their own row
-// with tcgen05.ld and run the epilogue while the next tile's MMAs proceed.  Ragged shapes (rows, N, K)
-// rely on TMA zero fill plus store masks.  Every mbarrier wait is bounded.
+// CTA tile 128 rows x 256 or 128 output features (prefill_tc_split chooses per launch), K blocks of 64 (one 128-byte
+// swizzle span), same roles as the stacked LM head: warp 0 issues TMA loads into a shared-memory ring (3 stages of 64 KB or 4
+// of 48 KB), warp 1 issues tcgen05.mma into one of two 256-column accumulators in tensor memory, warps 2-9 read their own
+// row with tcgen05.ld, each half of the columns, and run the epilogue while the next tile's MMAs proceed.  A launch
+// with fewer tiles than half of the SMs (short prompts) cuts K into up to 4 parts: each CTA leaves its partial sums in the
+// workspace, takes a ticket, and the last one of a tile adds the parts in K order and runs the epilogue.
+// Ragged shapes (rows, N, K) rely on TMA zero fill plus store masks.  Every mbarrier wait is bounded.
 #include <cuda.h>
 
 #include "kernels.h"
@@ -31,24 +32,54 @@ namespace {
 
 using namespace tc;
 
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 3;
+constexpr int BM = 128, BK = 64, ACC = 256;      // ACC: columns of an accumulator
 // a stage: high parts of the activation tile, their low parts, the weight tile
-constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2, STAGE_BYTES = 2 * A_BYTES + B_BYTES;
-constexpr int PF_THREADS = 192;
-// O-proj and down (N = d_model) use a narrower tile, p.bn_narrow, chosen per model shape (prefill_tc_narrow)
-template <int EPI> __device__ __forceinline__ int tile_n(const PfArgs &p) {
-    return (EPI == PF_OPROJ || EPI == PF_DOWN) ? p.bn_narrow : BN;
-}
+constexpr int A_BYTES = BM * BK * 2, RING_BYTES = 3 * (2 * A_BYTES + 256 * BK * 2), MAX_STAGES = 4;
+constexpr int PF_THREADS = 320, EPI_WARPS = 8;
+static_assert(RING_BYTES == 4 * (2 * A_BYTES + 128 * BK * 2), "both tile widths fill the ring");
 
 struct PfMaps {
-    CUtensorMap a, a_lo;       // activations [PF_ROWS, K], high and low parts, box 64 x 128
-    CUtensorMap b0, b1, b2;    // weights [N, K]: QKV Wq / Wk / Wv (box 64 x 256); GATEUP gate / up (box 64 x 128); else b0
+    CUtensorMap a, a_lo;       // activations [chunk rows, K], high and low parts, box 64 x 128
+    CUtensorMap b0, b1, b2;    // weights [N, K]: QKV Wq / Wk / Wv (box 64 x 128); GATEUP gate / up (box 64 x 64); else b0 (64 x 128)
+};
+
+// where a tile's sums are: an accumulator in tensor memory, or the partial sums of a tile whose K was cut
+struct Sums {
+    uint32_t taddr;
+    const float *part;         // [parts][columns / 32][128 rows][32], this thread's row; nullptr: tensor memory
+    int parts, stride;         // floats between two parts
+    __device__ __forceinline__ void load32(int col, uint32_t (&r)[32]) const {
+        if (part == nullptr) {
+            tmem_ld32(taddr + (uint32_t)col, r);
+            return;
+        }
+        float s[32];
+#pragma unroll
+        for (int e = 0; e < 32; ++e) s[e] = 0.f;
+        const float *p = part + (size_t)(col >> 5) * BM * 32;
+        for (int i = 0; i < parts; ++i, p += stride)                  // ascending K
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float4 v = __ldcg(reinterpret_cast<const float4 *>(p) + e);
+                s[4 * e] += v.x; s[4 * e + 1] += v.y; s[4 * e + 2] += v.z; s[4 * e + 3] += v.w;
+            }
+#pragma unroll
+        for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(s[e]);
+    }
 };
 
 // 1/rms of a row from the producer's per-tile sums of squares
 __device__ __forceinline__ float row_rscale(const float *ssp, int n_part, int d, float eps) {
     float s = 0.f;
-    for (int i = 0; i < n_part; ++i) s += ldg_cg_f32(ssp + i);
+    if ((n_part & 3) == 0) {       // (then every row starts on 16 bytes)
+#pragma unroll 4
+        for (int i = 0; i < n_part; i += 4) {
+            const float4 v = __ldcg(reinterpret_cast<const float4 *>(ssp + i));
+            s = (((s + v.x) + v.y) + v.z) + v.w;
+        }
+    } else {
+        for (int i = 0; i < n_part; ++i) s += ldg_cg_f32(ssp + i);
+    }
     return rsqrtf(s / (float)d + eps);
 }
 
@@ -77,10 +108,51 @@ __device__ __forceinline__ void store_split_x32(bf16 *hi, bf16 *lo, const float 
     }
 }
 
-// ---- epilogues: one thread owns one row of the tile; taddr = this warp's lane quarter, accumulator column 0
+// Four entries of a rotary table.  Every lane reads another position's row, so an access costs as many passes through L1 as
+// lanes: 16 bytes at a time where the tables are aligned (the caller's pointers need not be) take a quarter of them
+// (7B shape, 1000 rows: the QKV launch 178 us with 4-byte loads, 165 with these).
+__device__ __forceinline__ void load_rope4(const float *q, int vec, float (&v)[4]) {
+    if (vec) {
+        const float4 f = __ldg(reinterpret_cast<const float4 *>(q));
+        v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = __ldg(q + i);
+    }
+}
+
+// 32 features of this lane's row, scaled and rounded to bf16, transposed among the 8 lanes of a block of rows: w[k] =
+// feature 8 k + (lane & 7) of the block's 8 rows
+__device__ __forceinline__ void transpose8(const uint32_t (&r)[32], float scale, bool live, int lane, uint4 (&w)[4]) {
+    uint32_t a[16], b[8][2];
+    const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const float x = live ? scale * __uint_as_float(r[2 * i]) : 0.f, y = live ? scale * __uint_as_float(r[2 * i + 1]) : 0.f;
+        const float got = __shfl_xor_sync(0xffffffffu, b0 ? x : y, 1);
+        a[i] = b0 ? pack_bf16(got, y) : pack_bf16(x, got);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t got = __shfl_xor_sync(0xffffffffu, b1 ? a[2 * i] : a[2 * i + 1], 2);
+        b[i][0] = b1 ? got : a[2 * i];
+        b[i][1] = b1 ? a[2 * i + 1] : got;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t g0 = __shfl_xor_sync(0xffffffffu, b2 ? b[2 * i][0] : b[2 * i + 1][0], 4);
+        const uint32_t g1 = __shfl_xor_sync(0xffffffffu, b2 ? b[2 * i][1] : b[2 * i + 1][1], 4);
+        w[i] = b2 ? make_uint4(g0, g1, b[2 * i + 1][0], b[2 * i + 1][1]) : make_uint4(b[2 * i][0], b[2 * i][1], g0, g1);
+    }
+}
+
+// ---- epilogues: one thread owns one row of the tile and, of its columns, the blocks of 32 (rotary and gate / up partners:
+// the pairs of blocks) with half = 0 the first, 1 the second half; rs: the row's 1/rms (QKV, GATEUP)
 template <int EPI>
-__device__ __forceinline__ void epilogue(const PfArgs &p, uint32_t taddr, int row, int nt) {
+__device__ __forceinline__ void epilogue(const PfArgs &p, const Sums &src, int row, int nt, int half_id, float rs) {
+    const int BN = p.bn;
     const bool live = row < p.M;
+    const int lane = threadIdx.x & 31;
     const Dims &D = p.D;
     uint32_t r0[32], r1[32];
     if (EPI == PF_QKV) {
@@ -89,26 +161,33 @@ __device__ __forceinline__ void epilogue(const PfArgs &p, uint32_t taddr, int ro
         const int which = nt < n_qt ? 0 : (nt < n_qt + n_kt ? 1 : 2);
         const int n0 = (nt - (which == 0 ? 0 : (which == 1 ? n_qt : n_qt + n_kt))) * BN;   // feature offset in its matrix
         const int n_out = which == 0 ? D.nh * hd : D.nkv * hd;
-        const float rs = live ? row_rscale(p.SSP + (size_t)row * p.n_ssp, p.n_ssp, D.d, D.eps) : 0.f;
-        const int pos = p.pos0 + (live ? row : 0);
+        const int pos = p.pos0 + min(row, p.M - 1);              // (rows past the chunk: the last live row's page)
         const int pg = p.PT[p.seq * D.pages_per_seq + (pos >> 4)], sl = pos & 15;
         if (which < 2) {
             const float *cs = p.rope_cos + (size_t)pos * half, *sn = p.rope_sin + (size_t)pos * half;
-            for (int h0 = 0; h0 < BN; h0 += hd) {                // heads inside the tile
-                for (int jj = 0; jj < half; jj += 32) {
+            const int per = half >> 5, n_pair = BN >> 6;             // pairs of blocks per head, per tile
+            for (int u = half_id * (n_pair >> 1); u < (half_id + 1) * (n_pair >> 1); ++u) {
+                {
+                    const int h0 = (per == 2 ? u >> 1 : u) * hd, jj = per == 2 ? (u & 1) * 32 : 0;     // head inside the tile
                     __syncwarp();
-                    tmem_ld32(taddr + (uint32_t)(h0 + jj), r0);
-                    tmem_ld32(taddr + (uint32_t)(h0 + half + jj), r1);
+                    src.load32(h0 + jj, r0);
+                    src.load32(h0 + half + jj, r1);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     const int n = n0 + h0;                       // first feature of the head
                     if (!live || n >= n_out) continue;
                     float lo[32], hi[32];
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        const float a = rs * __uint_as_float(r0[e]), b = rs * __uint_as_float(r1[e]);
-                        const float c = __ldg(cs + jj + e), s = __ldg(sn + jj + e);
-                        lo[e] = a * c - b * s;
-                        hi[e] = b * c + a * s;
+                    for (int e4 = 0; e4 < 32; e4 += 4) {
+                        float c[4], s[4];
+                        load_rope4(cs + jj + e4, p.rope_vec, c);
+                        load_rope4(sn + jj + e4, p.rope_vec, s);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int e = e4 + i;
+                            const float a = rs * __uint_as_float(r0[e]), b = rs * __uint_as_float(r1[e]);
+                            lo[e] = a * c[i] - b * s[i];
+                            hi[e] = b * c[i] + a * s[i];
+                        }
                     }
                     if (which == 0) {
                         const size_t qo = (size_t)row * (D.nh * hd) + n + jj;
@@ -122,28 +201,35 @@ __device__ __forceinline__ void epilogue(const PfArgs &p, uint32_t taddr, int ro
                 }
             }
         } else {
-            for (int c0 = 0; c0 < BN; c0 += 32) {
+            for (int c0 = half_id * (BN >> 1); c0 < (half_id + 1) * (BN >> 1); c0 += 32) {
                 __syncwarp();
-                tmem_ld32(taddr + (uint32_t)c0, r0);
+                src.load32(c0, r0);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (!live) continue;
+                const int n = n0 + c0;                           // 32 features of one head (n_out is a multiple of 64)
+                if (n >= n_out) continue;
+                const int kvh = n / hd, dim = n - kvh * hd;
+                if (p.vp_vec) {
+                    // transposed in blocks of 8 positions x 8 features across lanes: 4 stores of 16 bytes instead of 32 of 2
+                    // (positions past the prompt that share a block with it get zeros)
+                    uint4 w[4];
+                    transpose8(r0, live ? rs : 0.f, live, lane, w);
+                    if ((row & ~7) < p.M) {
+                        bf16 *dst = p.VP + ((((size_t)pg * D.L + (p.layer - 1)) * D.nkv + kvh) * hd + dim + (lane & 7)) * 16 + (sl & 8);
 #pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    const int n = n0 + c0 + e;
-                    if (n < n_out) {
-                        const int kvh = n / hd, dim = n - kvh * hd;
-                        p.VP[((((size_t)pg * D.L + (p.layer - 1)) * D.nkv + kvh) * hd + dim) * 16 + sl] =
-                            __float2bfloat16_rn(rs * __uint_as_float(r0[e]));
+                        for (int k = 0; k < 4; ++k) *reinterpret_cast<uint4 *>(dst + (size_t)k * 8 * 16) = w[k];
                     }
+                } else if (live) {
+                    bf16 *dst = p.VP + ((((size_t)pg * D.L + (p.layer - 1)) * D.nkv + kvh) * hd + dim) * 16 + sl;
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) dst[e * 16] = __float2bfloat16_rn(rs * __uint_as_float(r0[e]));
                 }
             }
         }
     } else if (EPI == PF_GATEUP) {
-        const float rs = live ? row_rscale(p.SSPM + (size_t)row * p.n_ssp, p.n_ssp, D.d, D.eps) : 0.f;
-        for (int c0 = 0; c0 < BN / 2; c0 += 32) {
+        for (int c0 = half_id * (BN >> 2); c0 < (half_id + 1) * (BN >> 2); c0 += 32) {
             __syncwarp();
-            tmem_ld32(taddr + (uint32_t)c0, r0);
-            tmem_ld32(taddr + (uint32_t)(BN / 2 + c0), r1);
+            src.load32(c0, r0);
+            src.load32(BN / 2 + c0, r1);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             const int f0 = nt * (BN / 2) + c0;
             if (!live || f0 >= D.F) continue;
@@ -163,11 +249,11 @@ __device__ __forceinline__ void epilogue(const PfArgs &p, uint32_t taddr, int ro
     } else {   // PF_OPROJ, PF_DOWN: residual update in place, next norm input, sums of squares of the new h
         float ss = 0.f;
         bf16 *xo = EPI == PF_OPROJ ? p.XM : p.XS, *xl = EPI == PF_OPROJ ? p.XML : p.XSL;
-        for (int c0 = 0; c0 < p.bn_narrow; c0 += 32) {
+        for (int c0 = half_id * (BN >> 1); c0 < (half_id + 1) * (BN >> 1); c0 += 32) {
             __syncwarp();
-            tmem_ld32(taddr + (uint32_t)c0, r0);
+            src.load32(c0, r0);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            const int n = nt * p.bn_narrow + c0;
+            const int n = nt * BN + c0;
             if (!live || n >= D.d) continue;                     // d is a multiple of 32
             float *hp = p.H + (size_t)row * D.d + n;
             float h[32];
@@ -193,9 +279,9 @@ __device__ __forceinline__ void epilogue(const PfArgs &p, uint32_t taddr, int ro
                 x[e] = p.gain ? h[e] * bf16_to_f(p.gain[n + e]) : 0.f;
             }
             if (p.gain) store_split_x32(xo + (size_t)row * D.d + n, xl + (size_t)row * D.d + n, x);
-            // one partial sum of squares per 128 columns, whatever the tile width: results do not depend on it
-            if ((c0 & 127) == 96 || n + 32 >= D.d) {
-                (EPI == PF_OPROJ ? p.SSPM : p.SSP)[(size_t)row * p.n_ssp + (n >> 7)] = ss;
+            // one partial sum of squares per 64 columns, whatever the tile width: results do not depend on it
+            if ((c0 & 63) == 32 || n + 32 >= D.d) {
+                (EPI == PF_OPROJ ? p.SSPM : p.SSP)[(size_t)row * p.n_ssp + (n >> 6)] = ss;
                 ss = 0.f;
             }
         }
@@ -205,16 +291,17 @@ __device__ __forceinline__ void epilogue(const PfArgs &p, uint32_t taddr, int ro
 template <int EPI>
 __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __grid_constant__ PfMaps maps, const PfArgs p) {
     extern __shared__ unsigned char smem_dyn[];
-    __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], tfull_bar[2], tempty_bar[2];
+    __shared__ __align__(8) uint64_t full_bar[MAX_STAGES], empty_bar[MAX_STAGES], tfull_bar[2], tempty_bar[2];
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int s_err;
+    __shared__ int s_last;
     // 1024-byte alignment for the 128-byte swizzle atoms
     unsigned char *tiles = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&tfull_bar[b], 1); mbar_init(&tempty_bar[b], 4); }
+        for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&tfull_bar[b], 1); mbar_init(&tempty_bar[b], EPI_WARPS); }
         s_err = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -230,57 +317,64 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
     pdl_launch();
     pdl_wait();
 
-    const int n_kb = (p.K + BK - 1) / BK;
+    const int bn = p.bn, n_stages = bn == 256 ? 3 : 4, b_bytes = bn * BK * 2, stage_bytes = 2 * A_BYTES + b_bytes;
+    const int n_kb_all = (p.K + BK - 1) / BK;
     const int n_mt = (p.M + BM - 1) / BM;
     const int n_tiles = n_mt * p.n_ntiles;
-    const int my_tiles = (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    // with K cut into parts every CTA has one (tile, part); otherwise tiles go round
+    const int part = p.k_parts > 1 ? (int)blockIdx.x / n_tiles : 0, tile0 = (int)blockIdx.x - part * n_tiles;
+    const int kb_first = n_kb_all * part / p.k_parts, n_kb = n_kb_all * (part + 1) / p.k_parts - kb_first;
+    const int my_tiles = p.k_parts > 1 ? 1 : (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
 
     if (warp == 0) {
         if (lane == 0) {
-            const int n_qt = (p.D.nh * p.D.hd + BN - 1) / BN, n_kt = (p.D.nkv * p.D.hd + BN - 1) / BN;
-            int it = 0;
+            const int n_qt = (p.D.nh * p.D.hd + bn - 1) / bn, n_kt = (p.D.nkv * p.D.hd + bn - 1) / bn;
+            int s = 0;
+            uint32_t phase = 1;
             for (int i = 0; i < my_tiles && !s_err; ++i) {
-                const int tile = blockIdx.x + i * gridDim.x;
+                const int tile = tile0 + i * gridDim.x;
                 const int nt = tile / n_mt, mt = tile - nt * n_mt;      // row tiles of one weight tile run together
-                for (int kb = 0; kb < n_kb; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    if (!mbar_wait(&empty_bar[s], ((it / STAGES) & 1) ^ 1)) { s_err = 1; break; }
-                    mbar_expect_tx(&full_bar[s], 2 * A_BYTES + tile_n<EPI>(p) * BK * 2);
-                    unsigned char *sa = tiles + (size_t)s * STAGE_BYTES;
+                const CUtensorMap *mb = &maps.b0;
+                int y = nt * bn;
+                if (EPI == PF_QKV) {
+                    mb = nt < n_qt ? &maps.b0 : (nt < n_qt + n_kt ? &maps.b1 : &maps.b2);
+                    y = (nt - (nt < n_qt ? 0 : (nt < n_qt + n_kt ? n_qt : n_qt + n_kt))) * bn;
+                }
+                for (int kb = kb_first; kb < kb_first + n_kb; ++kb) {
+                    if (!mbar_wait(&empty_bar[s], phase)) { s_err = 1; break; }
+                    mbar_expect_tx(&full_bar[s], stage_bytes);
+                    unsigned char *sa = tiles + (size_t)s * stage_bytes, *sb = sa + 2 * A_BYTES;
                     tma_load_2d(sa, &maps.a, kb * BK, mt * BM, &full_bar[s]);
                     tma_load_2d(sa + A_BYTES, &maps.a_lo, kb * BK, mt * BM, &full_bar[s]);
-                    sa += A_BYTES;               // the weight tile follows the two activation tiles
-                    if (EPI == PF_QKV) {
-                        if (nt < n_qt) tma_load_2d(sa + A_BYTES, &maps.b0, kb * BK, nt * BN, &full_bar[s]);
-                        else if (nt < n_qt + n_kt) tma_load_2d(sa + A_BYTES, &maps.b1, kb * BK, (nt - n_qt) * BN, &full_bar[s]);
-                        else tma_load_2d(sa + A_BYTES, &maps.b2, kb * BK, (nt - n_qt - n_kt) * BN, &full_bar[s]);
-                    } else if (EPI == PF_GATEUP) {
-                        // accumulator columns 0..127: gate rows of this tile, 128..255: the same rows of W_up
-                        tma_load_2d(sa + A_BYTES, &maps.b0, kb * BK, nt * (BN / 2), &full_bar[s]);
-                        tma_load_2d(sa + A_BYTES + B_BYTES / 2, &maps.b1, kb * BK, nt * (BN / 2), &full_bar[s]);
+                    if (EPI == PF_GATEUP) {
+                        // accumulator columns 0 .. bn/2 - 1: gate rows of this tile, bn/2 .. bn - 1: the same rows of W_up
+                        for (int r = 0; r < bn / 2; r += 64) {
+                            tma_load_2d(sb + r * 128, &maps.b0, kb * BK, nt * (bn / 2) + r, &full_bar[s]);
+                            tma_load_2d(sb + (bn / 2 + r) * 128, &maps.b1, kb * BK, nt * (bn / 2) + r, &full_bar[s]);
+                        }
                     } else {
-                        tma_load_2d(sa + A_BYTES, &maps.b0, kb * BK, nt * tile_n<EPI>(p), &full_bar[s]);
+                        for (int r = 0; r < bn; r += 128) tma_load_2d(sb + r * 128, mb, kb * BK, y + r, &full_bar[s]);
                     }
+                    if (++s == n_stages) { s = 0; phase ^= 1; }
                 }
             }
         }
     } else if (warp == 1) {
         if (lane == 0) {
             // instruction descriptor: fp32 accumulate, bf16 x bf16, both operands K-major, N = tile width, M = 128
-            const uint32_t idesc =
-                (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(tile_n<EPI>(p) >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-            int it = 0;
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+            int s = 0;
+            uint32_t phase = 0;
             for (int i = 0; i < my_tiles && !s_err; ++i) {
                 const int buf = i & 1;
                 if (!mbar_wait(&tempty_bar[buf], ((i >> 1) & 1) ^ 1)) { s_err = 2; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t d_tmem = tmem_base + (uint32_t)buf * BN;
+                const uint32_t d_tmem = tmem_base + (uint32_t)buf * ACC;
                 bool ok = true;
-                for (int kb = 0; kb < n_kb; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    if (!mbar_wait(&full_bar[s], (it / STAGES) & 1)) { s_err = 3; ok = false; break; }
+                for (int kb = 0; kb < n_kb; ++kb) {
+                    if (!mbar_wait(&full_bar[s], phase)) { s_err = 3; ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t sa = smem_u32(tiles + (size_t)s * STAGE_BYTES);
+                    const uint32_t sa = smem_u32(tiles + (size_t)s * stage_bytes);
                     const uint64_t da = umma_desc(sa), dl = umma_desc(sa + A_BYTES), db = umma_desc(sa + 2 * A_BYTES);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k) {
@@ -288,20 +382,55 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
                         umma_bf16(d_tmem, dl + 2 * k, db + 2 * k, idesc, 1u);
                     }
                     umma_commit(&empty_bar[s]);      // the stage may be refilled once these MMAs have read it
+                    if (++s == n_stages) { s = 0; phase ^= 1; }
                 }
                 if (!ok) break;
                 umma_commit(&tfull_bar[buf]);        // accumulator complete
             }
         }
     } else {
-        const int q = warp & 3;                      // TMEM lane quarter this warp may read
+        const int q = warp & 3, half_id = (warp - 2) >> 2;   // TMEM lane quarter this warp may read, half of the columns
         for (int i = 0; i < my_tiles; ++i) {
-            const int tile = blockIdx.x + i * gridDim.x;
+            const int tile = tile0 + i * gridDim.x;
             const int nt = tile / n_mt, mt = tile - nt * n_mt;
-            const int buf = i & 1;
-            if (s_err || !mbar_wait(&tfull_bar[buf], (i >> 1) & 1)) { if (!s_err) s_err = 4; break; }
+            const int buf = i & 1, rr = q * 32 + lane, row = mt * BM + rr;
+            float rs = 0.f;
+            if ((EPI == PF_QKV || EPI == PF_GATEUP) && row < p.M)
+                rs = row_rscale((EPI == PF_QKV ? p.SSP : p.SSPM) + (size_t)row * p.n_ssp, p.n_ssp, p.D.d, p.D.eps);
+            bool ok = !s_err;
+            if (ok && !mbar_wait(&tfull_bar[buf], (i >> 1) & 1)) { s_err = 4; ok = false; }
+            if (p.k_parts == 1 && !ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            epilogue<EPI>(p, tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN), mt * BM + q * 32 + lane, nt);
+            Sums src{tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * ACC), nullptr, 1, 0};
+            if (p.k_parts > 1) {
+                // this part's sums -> workspace; the last of the tile's CTAs goes on
+                const int tile_floats = BM * bn;
+                if (ok) {
+                    float *o = p.part + ((size_t)part * n_tiles + tile) * tile_floats + rr * 32;
+                    for (int c0 = half_id * (bn >> 1); c0 < (half_id + 1) * (bn >> 1); c0 += 32) {
+                        uint32_t r[32];
+                        __syncwarp();
+                        tmem_ld32(src.taddr + (uint32_t)c0, r);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                        uint4 *d = reinterpret_cast<uint4 *>(o + (size_t)(c0 >> 5) * BM * 32);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) __stcg(d + e, make_uint4(r[4 * e], r[4 * e + 1], r[4 * e + 2], r[4 * e + 3]));
+                    }
+                }
+                asm volatile("bar.sync 1, 256;" ::: "memory");
+                if (threadIdx.x == 64) {
+                    int old = -1;
+                    if (!s_err) asm volatile("atom.add.acq_rel.gpu.s32 %0, [%1], 1;" : "=r"(old) : "l"(p.ticket + tile) : "memory");
+                    s_last = old == p.k_parts - 1;
+                    if (old == p.k_parts - 1) p.ticket[tile] = 0;
+                }
+                asm volatile("bar.sync 1, 256;" ::: "memory");
+                if (!s_last) break;
+                src.part = p.part + (size_t)tile * tile_floats + rr * 32;
+                src.parts = p.k_parts;
+                src.stride = n_tiles * tile_floats;
+            }
+            epilogue<EPI>(p, src, row, nt, half_id, rs);
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty_bar[buf]);
@@ -335,24 +464,24 @@ __global__ void __launch_bounds__(256) prefill_embed_kernel(const PfArgs p, cons
     ss = warp_sum(ss);
     if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = ss;
     __syncthreads();
-    if (threadIdx.x < p.n_ssp) {
+    for (int i = threadIdx.x; i < p.n_ssp; i += 256) {
         float t = 0.f;
-        if (threadIdx.x == 0)
+        if (i == 0)
             for (int w = 0; w < 8; ++w) t += s_red[w];
-        p.SSP[(size_t)row * p.n_ssp + threadIdx.x] = t;
+        p.SSP[(size_t)row * p.n_ssp + i] = t;
     }
 }
 
 template <int EPI>
 cudaError_t launch_epi(const PfMaps &maps, const PfArgs &p, int n_sms, cudaStream_t st, bool pdl) {
-    const size_t smem = (size_t)STAGES * STAGE_BYTES + 1024;
+    const size_t smem = (size_t)RING_BYTES + 1024;
     auto kern = prefill_gemm_kernel<EPI>;
     static SmemAttrOnce attr;
     {
         cudaError_t e = attr.set(kern, (int)((int)smem));
         if (e != cudaSuccess) return e;
     }
-    const int n_tiles = ((p.M + BM - 1) / BM) * p.n_ntiles;
+    const int n_tiles = ((p.M + BM - 1) / BM) * p.n_ntiles * p.k_parts;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_tiles < n_sms ? n_tiles : n_sms);
     cfg.blockDim = dim3(PF_THREADS);
@@ -368,36 +497,47 @@ cudaError_t launch_epi(const PfMaps &maps, const PfArgs &p, int n_sms, cudaStrea
 
 }  // namespace
 
-int prefill_tc_ntiles(int epi, const Dims &D) {
+int prefill_tc_nssp(const Dims &D) { return (D.d + 63) / 64; }
+
+namespace {
+
+int n_tiles_of(int epi, const Dims &D, int bn) {
     switch (epi) {
-        case PF_QKV: return (D.nh * D.hd + BN - 1) / BN + 2 * ((D.nkv * D.hd + BN - 1) / BN);
-        case PF_GATEUP: return (D.F + BN / 2 - 1) / (BN / 2);
-        default: { const int bn = prefill_tc_narrow(D); return (D.d + bn - 1) / bn; }
+        case PF_QKV: return (D.nh * D.hd + bn - 1) / bn + 2 * ((D.nkv * D.hd + bn - 1) / bn);
+        case PF_GATEUP: return (D.F + bn / 2 - 1) / (bn / 2);
+        default: return (D.d + bn - 1) / bn;
     }
 }
-int prefill_tc_nssp(const Dims &D) { return (D.d + 127) / 128; }
 
-// Tile width of the two GEMMs whose N is d_model: 128 or 256 (whole 128-column groups of the per-row sums of
-// squares, so that no result depends on the choice).  A k-block of a 128 x bn tile costs its operand loads,
-// (128 + bn) rows of 128 bytes at what one SM can pull from L2, more than its MMAs (measured: tensor pipe 40-68 %
-// active), so a tile takes about (128 + bn) units; the width that minimises waves x (128 + bn) for a full chunk
-// of PF_ROWS rows on 148 SMs wins: 128 at d = 4096 (128 tiles, one wave), 256 at d = 5120 (80 tiles in one wave
-// instead of 160 in two: the 3072-position prefill of that shape 138 -> 127 ms).
-int prefill_tc_narrow(const Dims &D) {
-    int best = 128;
-    long best_cost = -1;
-    for (int bn = 128; bn <= 256; bn += 128) {
-        const long tiles = (long)(PF_ROWS / BM) * ((D.d + bn - 1) / bn);
-        const long cost = ((tiles + 147) / 148) * (128 + bn);
-        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = bn; }
-    }
-    return best;
+// Tile width and parts of K of a launch: the choice with the smallest estimated time, waves of tiles on the SMs x (K blocks of
+// a tile x what a block takes + the epilogue of the last tile) + the merge of the parts; the constants are microseconds that
+// reproduce the measured launches.  Measured (us, 256 wide / 128 wide / 128 wide with K in parts):
+//   7B shape,   96 rows: O 55 / 37 / 33,   down 119 / 80 / 45 (4 parts),   gate/up 55 / 68
+//   7B shape,  160 rows: O 60 / 39 / 36,   down 123 / 82 / 58 (2 parts),   gate/up 94 / 98
+//   7B shape,  512 rows: O 61 / 41,        down 127 / 87,                  gate/up 143 / 164
+//   7B shape, 1000 rows: O 63 / 69,        down 141 / 167,                 gate/up 234 / 308
+//   13B shape, 1024 rows: O 131 / 119,     down 327 / 314 (the model says 256 for down),   gate/up 363 / 472
+void choose_split(int epi, int n_sms, PfArgs &p) {
+    const int n_mt = (p.M + BM - 1) / BM, n_kb = (p.K + BK - 1) / BK;
+    double best = 0.0;
+    for (int bn = 256; bn >= 128; bn -= 128)
+        for (int parts = 1; parts <= (bn == 128 ? 4 : 1); ++parts) {
+            const int nt = n_tiles_of(epi, p.D, bn), tiles = n_mt * nt;
+            if (parts > 1 && (tiles * parts > n_sms || tiles * parts > DEL_WT_CTAS || n_kb < 4 * parts)) continue;
+            const double t = (tiles * parts + n_sms - 1) / n_sms * ((double)n_kb / parts * (bn == 256 ? 0.70 : 0.45)) + (bn == 256 ? 8 : 4) + (parts > 1 ? 3 + parts : 0);
+            if (best == 0.0 || t < best) { best = t; p.bn = bn; p.n_ntiles = nt; p.k_parts = parts; }
+        }
 }
 
-// map_a / map_b*: 128-byte CUtensorMap blobs made by lmhead_tc_make_map (boxes of 256 rows for Wq / Wk / Wv, of
-// 128 rows for the activations and for W_gate / W_up / W_o / W_down)
+}  // namespace
+
+// map_a / map_b*: 128-byte CUtensorMap blobs made by lmhead_tc_make_map (boxes of 128 rows, W_gate / W_up 64)
 cudaError_t launch_prefill_gemm(int epi, const void *map_a, const void *map_a_lo, const void *map_b0, const void *map_b1,
-                                const void *map_b2, const PfArgs &p, int n_sms, cudaStream_t st, bool pdl) {
+                                const void *map_b2, const PfArgs &args, int n_sms, cudaStream_t st, bool pdl) {
+    PfArgs p = args;
+    choose_split(epi, n_sms, p);
+    p.rope_vec = ((reinterpret_cast<uintptr_t>(p.rope_cos) | reinterpret_cast<uintptr_t>(p.rope_sin)) & 15) == 0;      // rows are whole multiples of 16 bytes
+    p.vp_vec = (reinterpret_cast<uintptr_t>(p.VP) & 15) == 0;
     PfMaps maps;
     maps.a = *reinterpret_cast<const CUtensorMap *>(map_a);
     maps.a_lo = *reinterpret_cast<const CUtensorMap *>(map_a_lo);

@@ -57,3 +57,25 @@ def test_rounds_against_oracle(batch, g_max):
         assert rep.ok(), (s, rep.failures[:5])
         assert rep.rounds == len(refs[s].rounds)
     ctx.close()
+
+
+@pytest.mark.parametrize("prompt_len", [40, 47, 63, 65, 129, 200, 257, 1023, 1030, 1050])
+@pytest.mark.parametrize("cfg", [RAGGED, HD128], ids=lambda c: c.name)
+def test_prompt_kernels_against_decode_kernels(cfg, prompt_len):
+    """Prompts around the shortest the prefill kernels take, ragged last row tiles, K in parts (few tiles), two chunks of
+    positions and a window that straddles them: cache and hidden states against the decode kernels.  Those round queries
+    and probabilities to bf16 (2^-9 each), the prefill kernels do not: 2^-7 of a vector's norm."""
+    import paper_2504_05598_b200 as dl
+    cfg = synth.small_variant(cfg, prompt_len=prompt_len, gen_len=4)
+    w = synth.make_weights(cfg)
+    ctx = make_ctx(cfg, w)
+    got = []
+    for more in (0, dl.FLAG_NO_BULK_PREFILL):
+        ctx.set_flags(dl.FLAG_PDL | dl.FLAG_TC | more)
+        ctx.prefill(0, synth.make_prompt(cfg), 2)
+        at = sorted({0, 7, 8, 15, 16, prompt_len // 2, prompt_len - 17, prompt_len - 2, prompt_len - 1} | set(range(1020, min(1030, prompt_len))))
+        got.append([ctx.get_hidden(0, l, j) for l in range(cfg.n_layers + 1) for j in (0, 13, 31)] +
+                   [x for l in range(1, cfg.n_layers + 1) for pos in at for x in ctx.get_kv(0, l, pos)])
+    for a, b in zip(*got):
+        assert np.linalg.norm(a - b) <= 2.0 ** -7 * np.linalg.norm(b)
+    ctx.close()
