@@ -725,13 +725,14 @@ int draft_with_exit(del_ctx *c, std::vector<Job> &jobs) {
 
 // ---- a whole prompt (positions 0 .. n_pos-1 of sequence sq) through the tensor-core GEMMs: the KV cache of
 // every position, and every layer's hidden state of the positions from win0 on (the window that seeds the
-// statistics) into the hidden stack; chunks of PF_ROWS positions, attention in passes of DEL_ROWS_MAX query rows
+// statistics) into the hidden stack; chunks of at most PF_ROWS positions, attention in passes of DEL_ROWS_MAX query rows
 int prefill_bulk(del_ctx *c, int sq, int n_pos, int win0) {
     const Dims &D = c->D;
     const bool P = pdl(c);
-    for (int p0 = 0; p0 < n_pos; p0 += PF_ROWS) {
+    const int chunk = prefill_tc_chunk(D, n_pos, c->n_sms, prefill_rows(c->sh));
+    for (int p0 = 0; p0 < n_pos; p0 += chunk) {
         PfArgs a = c->pf;
-        a.M = std::min(PF_ROWS, n_pos - p0);
+        a.M = std::min(chunk, n_pos - p0);
         a.seq = sq;
         a.pos0 = p0;
         a.stackH = c->B.H;

@@ -175,10 +175,10 @@ cudaError_t launch_lmhead_tc(const void *map_x, const void *map_w, float *part_v
 
 // Prompt prefill on tcgen05 (prefill_tc.cu): tiled GEMMs over up to PF_ROWS prompt positions of one sequence
 // with the layer's element-wise work fused into the epilogues.  All buffers hold PF_ROWS rows (fewer if max_seq is smaller).
-// 1024 rather than 512: twice the tiles leave less of the last wave of tiles idle (7B shape, 1000 positions: gate/up 5 waves
-// instead of 3 + 3, QKV 3 instead of 2 + 2; 860 -> 679 us per layer), while a chunk's activations (57 MB for the 13B
-// shape's down projection) still fit L2 beside the weights in flight.
-#define PF_ROWS 1024
+// prefill_tc_chunk picks the rows of a chunk up to this.  More rows leave less of a launch's last wave of tiles idle (7B
+// shape, 1000 positions: gate/up 5 waves in one chunk, 3 + 3 in two of 512, QKV 3 and 2 + 2: 679 and 860 us per layer); with
+// 2048 the widest activations (113 MB for the 13B shape's down projection) still about fit L2.
+#define PF_ROWS 2048
 enum { PF_QKV = 0, PF_OPROJ = 1, PF_GATEUP = 2, PF_DOWN = 3 };
 struct PfArgs {
     Dims D;
@@ -206,6 +206,7 @@ struct PfArgs {
     float *stackH;
     int32_t win0;
 };
+int prefill_tc_chunk(const Dims &D, int n, int n_sms, int max_rows);
 int prefill_tc_nssp(const Dims &D);            // partial sums of squares per row
 
 // Causal attention of a prefill chunk (prefill_attn.cu): rows 0..M-1 of Q (positions pos0 + row of sequence seq)

@@ -25,6 +25,8 @@
 // Ragged shapes (rows, N, K) rely on TMA zero fill plus store masks.  Every mbarrier wait is bounded.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "kernels.h"
 #include "tc_common.cuh"
 
@@ -94,17 +96,30 @@ __device__ __forceinline__ void store_bf16x32(bf16 *dst, const float (&v)[32]) {
         *reinterpret_cast<uint4 *>(dst + 8 * q) = w;
     }
 }
-// the same values as high parts to `hi` and low parts to `lo`
+// Whole 32-byte sectors per lane: the lanes' rows are far apart, so a 16-byte store writes half of a sector, and the other
+// half is a second transaction (7B shape, 1000 rows, us: O-projection 63 -> 57, down 136 -> 130)
+__device__ __forceinline__ void store32(void *dst, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e, uint32_t f, uint32_t g, uint32_t h) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(a), "r"(b), "r"(c), "r"(d), "r"(e), "r"(f), "r"(g), "r"(h) : "memory");
+}
+__device__ __forceinline__ void load32(const float *src, float *v) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(src) : "memory");
+}
+__device__ __forceinline__ void store_f32x32(float *dst, const float (&v)[32]) {
+#pragma unroll
+    for (int q = 0; q < 32; q += 8)
+        store32(dst + q, __float_as_uint(v[q]), __float_as_uint(v[q + 1]), __float_as_uint(v[q + 2]), __float_as_uint(v[q + 3]),
+                __float_as_uint(v[q + 4]), __float_as_uint(v[q + 5]), __float_as_uint(v[q + 6]), __float_as_uint(v[q + 7]));
+}
+// the same values as high parts to `hi` and low parts to `lo` (both 32-byte aligned: rows of the workspace)
 __device__ __forceinline__ void store_split_x32(bf16 *hi, bf16 *lo, const float (&v)[32]) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        uint4 wh, wl;
-        split_bf16x2(v[8 * q + 0], v[8 * q + 1], wh.x, wl.x);
-        split_bf16x2(v[8 * q + 2], v[8 * q + 3], wh.y, wl.y);
-        split_bf16x2(v[8 * q + 4], v[8 * q + 5], wh.z, wl.z);
-        split_bf16x2(v[8 * q + 6], v[8 * q + 7], wh.w, wl.w);
-        *reinterpret_cast<uint4 *>(hi + 8 * q) = wh;
-        *reinterpret_cast<uint4 *>(lo + 8 * q) = wl;
+    for (int q = 0; q < 32; q += 16) {
+        uint32_t wh[8], wl[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) split_bf16x2(v[q + 2 * i], v[q + 2 * i + 1], wh[i], wl[i]);
+        store32(hi + q, wh[0], wh[1], wh[2], wh[3], wh[4], wh[5], wh[6], wh[7]);
+        store32(lo + q, wl[0], wl[1], wl[2], wl[3], wl[4], wl[5], wl[6], wl[7]);
     }
 }
 
@@ -258,20 +273,12 @@ __device__ __forceinline__ void epilogue(const PfArgs &p, const Sums &src, int r
             float *hp = p.H + (size_t)row * D.d + n;
             float h[32];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const float4 v = *reinterpret_cast<const float4 *>(hp + 4 * q);
-                h[4 * q + 0] = v.x + __uint_as_float(r0[4 * q + 0]);
-                h[4 * q + 1] = v.y + __uint_as_float(r0[4 * q + 1]);
-                h[4 * q + 2] = v.z + __uint_as_float(r0[4 * q + 2]);
-                h[4 * q + 3] = v.w + __uint_as_float(r0[4 * q + 3]);
-                *reinterpret_cast<float4 *>(hp + 4 * q) = make_float4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
-            }
-            if (EPI == PF_DOWN && p.pos0 + row >= p.win0) {
-                float *sp = p.stackH + stack_row(D, p.layer, p.seq, p.pos0 + row - p.win0) * D.d + n;
+            for (int q = 0; q < 32; q += 8) load32(hp + q, h + q);
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    *reinterpret_cast<float4 *>(sp + 4 * q) = make_float4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
-            }
+            for (int e = 0; e < 32; ++e) h[e] += __uint_as_float(r0[e]);
+            store_f32x32(hp, h);
+            if (EPI == PF_DOWN && p.pos0 + row >= p.win0)
+                store_f32x32(p.stackH + stack_row(D, p.layer, p.seq, p.pos0 + row - p.win0) * D.d + n, h);
             float x[32];
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
@@ -517,25 +524,49 @@ int n_tiles_of(int epi, const Dims &D, int bn) {
 //   7B shape,  512 rows: O 61 / 41,        down 127 / 87,                  gate/up 143 / 164
 //   7B shape, 1000 rows: O 63 / 69,        down 141 / 167,                 gate/up 234 / 308
 //   13B shape, 1024 rows: O 131 / 119,     down 327 / 314 (the model says 256 for down),   gate/up 363 / 472
-void choose_split(int epi, int n_sms, PfArgs &p) {
-    const int n_mt = (p.M + BM - 1) / BM, n_kb = (p.K + BK - 1) / BK;
-    double best = 0.0;
+struct Split { int bn, parts; double us; };
+Split choose_split(int epi, const Dims &D, int M, int n_sms) {
+    const int K = epi == PF_OPROJ ? D.nh * D.hd : (epi == PF_DOWN ? D.F : D.d);
+    const int n_mt = (M + BM - 1) / BM, n_kb = (K + BK - 1) / BK;
+    Split best{0, 0, 0.0};
     for (int bn = 256; bn >= 128; bn -= 128)
         for (int parts = 1; parts <= (bn == 128 ? 4 : 1); ++parts) {
-            const int nt = n_tiles_of(epi, p.D, bn), tiles = n_mt * nt;
-            if (parts > 1 && (tiles * parts > n_sms || tiles * parts > DEL_WT_CTAS || n_kb < 4 * parts)) continue;
-            const double t = (tiles * parts + n_sms - 1) / n_sms * ((double)n_kb / parts * (bn == 256 ? 0.70 : 0.45)) + (bn == 256 ? 8 : 4) + (parts > 1 ? 3 + parts : 0);
-            if (best == 0.0 || t < best) { best = t; p.bn = bn; p.n_ntiles = nt; p.k_parts = parts; }
+            const int tiles = n_mt * n_tiles_of(epi, D, bn) * parts;
+            if (parts > 1 && (tiles > n_sms || tiles > DEL_WT_CTAS || n_kb < 4 * parts)) continue;
+            const double us = (tiles + n_sms - 1) / n_sms * ((double)n_kb / parts * (bn == 256 ? 0.70 : 0.45)) + (bn == 256 ? 8 : 4) + (parts > 1 ? 3 + parts : 0);
+            if (best.bn == 0 || us < best.us) best = Split{bn, parts, us};
         }
+    return best;
 }
 
 }  // namespace
+
+// Positions per chunk of a prompt of n: the whole number of 128-row tiles, at most max_rows, with the smallest estimated
+// time of the four GEMMs over all chunks (a wave of tiles that is nearly empty costs as much as a full one: the 13B shape's
+// down projection has 160 tiles of 256 at 1024 rows, 240 at 1536, on 148 SMs; its 3072-position prompt
+// takes 3418 us per layer in chunks of 1024 and 2742 in chunks of 1536)
+int prefill_tc_chunk(const Dims &D, int n, int n_sms, int max_rows) {
+    int best = 0;
+    double best_us = 0.0;
+    for (int c = std::min((n + BM - 1) / BM * BM, max_rows / BM * BM); c >= BM; c -= BM) {
+        double us = 0.0;
+        for (int p = 0; p < n; p += c) {
+            us += 10.0;                                                 // launches, the attention's ragged blocks
+            for (int epi = PF_QKV; epi <= PF_DOWN; ++epi) us += choose_split(epi, D, std::min(c, n - p), n_sms).us;
+        }
+        if (best == 0 || us < best_us) { best = c; best_us = us; }
+    }
+    return best;
+}
 
 // map_a / map_b*: 128-byte CUtensorMap blobs made by lmhead_tc_make_map (boxes of 128 rows, W_gate / W_up 64)
 cudaError_t launch_prefill_gemm(int epi, const void *map_a, const void *map_a_lo, const void *map_b0, const void *map_b1,
                                 const void *map_b2, const PfArgs &args, int n_sms, cudaStream_t st, bool pdl) {
     PfArgs p = args;
-    choose_split(epi, n_sms, p);
+    const Split s = choose_split(epi, p.D, p.M, n_sms);
+    p.bn = s.bn;
+    p.k_parts = s.parts;
+    p.n_ntiles = n_tiles_of(epi, p.D, s.bn);
     p.rope_vec = ((reinterpret_cast<uintptr_t>(p.rope_cos) | reinterpret_cast<uintptr_t>(p.rope_sin)) & 15) == 0;      // rows are whole multiples of 16 bytes
     p.vp_vec = (reinterpret_cast<uintptr_t>(p.VP) & 15) == 0;
     PfMaps maps;

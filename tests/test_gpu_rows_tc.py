@@ -59,7 +59,7 @@ def test_rounds_against_oracle(batch, g_max):
     ctx.close()
 
 
-@pytest.mark.parametrize("prompt_len", [40, 47, 63, 65, 129, 200, 257, 1023, 1030, 1050])
+@pytest.mark.parametrize("prompt_len", [40, 47, 63, 65, 129, 200, 257, 1030, 2047, 2060, 2075])
 @pytest.mark.parametrize("cfg", [RAGGED, HD128], ids=lambda c: c.name)
 def test_prompt_kernels_against_decode_kernels(cfg, prompt_len):
     """Prompts around the shortest the prefill kernels take, ragged last row tiles, K in parts (few tiles), two chunks of
@@ -73,7 +73,8 @@ def test_prompt_kernels_against_decode_kernels(cfg, prompt_len):
     for more in (0, dl.FLAG_NO_BULK_PREFILL):
         ctx.set_flags(dl.FLAG_PDL | dl.FLAG_TC | more)
         ctx.prefill(0, synth.make_prompt(cfg), 2)
-        at = sorted({0, 7, 8, 15, 16, prompt_len // 2, prompt_len - 17, prompt_len - 2, prompt_len - 1} | set(range(1020, min(1030, prompt_len))))
+        at = sorted({0, 7, 8, 15, 16, prompt_len // 2, prompt_len - 17, prompt_len - 2, prompt_len - 1} |
+                    {x for b in (1536, 2048) for x in range(b - 3, b + 4) if x < prompt_len})
         got.append([ctx.get_hidden(0, l, j) for l in range(cfg.n_layers + 1) for j in (0, 13, 31)] +
                    [x for l in range(1, cfg.n_layers + 1) for pos in at for x in ctx.get_kv(0, l, pos)])
     for a, b in zip(*got):
