@@ -272,6 +272,11 @@ int del_get_kv(del_ctx *ctx, int seq, int layer, int pos, float *k_out, float *v
  * an expired wait would have: a test hook for the error path that makes no kernel wait. */
 int del_debug_inject_error(del_ctx *ctx, int code);
 
+/* Test reader, host arithmetic only (no context, no GPU): the kernels a shape's passes take on a device with n_sms SMs.
+ * out (HOST int32 [10]): [0] rows from which on a layer pass takes the tcgen05 GEMMs (65: never); [1] positions per chunk of
+ * a prompt of n_prompt; then tile width and parts of K of the prefill GEMMs QKV, O, gate/up and down over `rows` positions. */
+int del_debug_routes(const del_shape *shape, int n_sms, int n_prompt, int rows, int32_t *out);
+
 /* Committed length (prompt + emitted tokens) of a sequence, or a negative code. */
 int del_committed_len(del_ctx *ctx, int seq);
 /* Frees the sequence's KV pages and marks it empty. */

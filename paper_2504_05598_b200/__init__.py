@@ -29,7 +29,7 @@ EXPORTS = ["del_workspace_bytes", "del_init", "del_prefill", "del_draft", "del_v
            "del_select", "del_round", "del_set_policy", "del_get_stats", "del_set_stats", "del_get_shadow",
            "del_get_drafts", "del_force_token", "del_get_hidden", "del_debug_logits", "del_get_kv", "del_committed_len", "del_release",
            "del_launch_count", "del_get_traffic", "del_set_flags", "del_get_kernel_times", "del_head_argmax_static",
-           "del_set_policy_fs", "del_set_exit_mode", "del_get_window", "del_set_sampling", "del_get_sample_info", "del_get_round_logits", "del_sample_probe", "del_get_conf_stats", "del_set_conf_stats", "del_get_conf", "del_debug_inject_error", "del_strerror", "del_last_cuda_error", "del_destroy"]
+           "del_set_policy_fs", "del_set_exit_mode", "del_get_window", "del_set_sampling", "del_get_sample_info", "del_get_round_logits", "del_sample_probe", "del_get_conf_stats", "del_set_conf_stats", "del_get_conf", "del_debug_inject_error", "del_debug_routes", "del_strerror", "del_last_cuda_error", "del_destroy"]
 
 
 class Shape(C.Structure):
@@ -131,6 +131,8 @@ def load_library(build_if_missing: bool = True):
     L.del_get_kv.argtypes = [vp, ci, ci, ci, vp, vp]
     L.del_debug_inject_error.restype = ci
     L.del_debug_inject_error.argtypes = [vp, ci]
+    L.del_debug_routes.restype = ci
+    L.del_debug_routes.argtypes = [C.POINTER(Shape), ci, ci, ci, C.POINTER(i32)]
     L.del_committed_len.restype = ci
     L.del_committed_len.argtypes = [vp, ci]
     L.del_release.restype = ci
@@ -410,6 +412,15 @@ class DelContext:
 
     def set_flags(self, flags: int) -> int:
         return self.lib.del_set_flags(self._h, flags)
+
+
+def debug_routes(shape: Shape, n_sms: int, n_prompt: int, rows: int):
+    """(rows_min, chunk, [(tile width, parts of K) of QKV, O, gate/up, down]) of del_debug_routes."""
+    out = (C.c_int32 * 10)()
+    rc = load_library().del_debug_routes(C.byref(shape), n_sms, n_prompt, rows, out)
+    if rc != OK:
+        raise DelError(rc, "del_debug_routes")
+    return out[0], out[1], [(out[2 + 2 * i], out[3 + 2 * i]) for i in range(4)]
 
 
 def upload_weights(w, device="cuda:0") -> Dict:

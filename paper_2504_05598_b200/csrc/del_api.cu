@@ -1043,6 +1043,21 @@ size_t del_workspace_bytes(const del_shape *shape) {
     return carve_all(*shape, nullptr, D, B, R, nv, &o, &dbg, nullptr, nullptr);
 }
 
+int del_debug_routes(const del_shape *shape, int n_sms, int n_prompt, int rows, int32_t *out) {
+    if (validate(shape) != DEL_OK || n_sms < 1 || n_prompt < 1 || rows < 1 || !out) return DEL_EINVAL;
+    Dims D; Buffers B; int R, nv; del_round_out *o; float *dbg;
+    carve_all(*shape, nullptr, D, B, R, nv, &o, &dbg, nullptr, nullptr);
+    out[0] = rowgemm_tc_supported(D) ? rows_min_tc(D) : DEL_ROWS_MAX + 1;
+    out[1] = prefill_tc_chunk(D, n_prompt, n_sms, prefill_rows(*shape));
+    for (int epi = PF_QKV; epi <= PF_DOWN; ++epi) {
+        int bn, parts;
+        prefill_tc_split(epi, D, rows, n_sms, &bn, &parts);
+        out[2 + 2 * epi] = bn;
+        out[3 + 2 * epi] = parts;
+    }
+    return DEL_OK;
+}
+
 int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const del_kv *kv, void *workspace,
              size_t ws_bytes, void *cuda_stream) {
     if (!out || !w || !kv || !workspace) return DEL_EINVAL;

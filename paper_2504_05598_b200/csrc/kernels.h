@@ -207,6 +207,7 @@ struct PfArgs {
     int32_t win0;
 };
 int prefill_tc_chunk(const Dims &D, int n, int n_sms, int max_rows);
+void prefill_tc_split(int epi, const Dims &D, int M, int n_sms, int *bn, int *parts);      // what launch_prefill_gemm chooses
 int prefill_tc_nssp(const Dims &D);            // partial sums of squares per row
 
 // Causal attention of a prefill chunk (prefill_attn.cu): rows 0..M-1 of Q (positions pos0 + row of sequence seq)

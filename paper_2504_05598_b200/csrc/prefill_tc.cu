@@ -517,13 +517,16 @@ int n_tiles_of(int epi, const Dims &D, int bn) {
 }
 
 // Tile width and parts of K of a launch: the choice with the smallest estimated time, waves of tiles on the SMs x (K blocks of
-// a tile x what a block takes + the epilogue of the last tile) + the merge of the parts; the constants are microseconds that
-// reproduce the measured launches.  Measured (us, 256 wide / 128 wide / 128 wide with K in parts):
-//   7B shape,   96 rows: O 55 / 37 / 33,   down 119 / 80 / 45 (4 parts),   gate/up 55 / 68
-//   7B shape,  160 rows: O 60 / 39 / 36,   down 123 / 82 / 58 (2 parts),   gate/up 94 / 98
-//   7B shape,  512 rows: O 61 / 41,        down 127 / 87,                  gate/up 143 / 164
-//   7B shape, 1000 rows: O 63 / 69,        down 141 / 167,                 gate/up 234 / 308
-//   13B shape, 1024 rows: O 131 / 119,     down 327 / 314 (the model says 256 for down),   gate/up 363 / 472
+// a tile x what a block takes) + the last tile's epilogue + the merge of the parts.  The constants are microseconds fitted to 897
+// launches of six layer shapes (50 to 635 MB) at 48 to 2048 rows: 6 % rms, and no launch whose choice is more than 7 % slower
+// than the best of the five.  Measured, us, 256 wide / 128 wide / 128 wide with K in 2, 3, 4 parts:
+//   7B shape,   48 rows: QKV 50 / 35,  O 49 / 34 / 30, 29, 29,  gate/up 53 / 64,  down 113 / 77 / 53, 44, 42
+//   7B shape,  160 rows: QKV 55 / 61,  O 53 / 36 / 34,          gate/up 92 / 90,  down 115 / 79 / 57
+//   7B shape,  512 rows: QKV 89 / 92,  O 54 / 39,               gate/up 137 / 154, down 118 / 87
+//   7B shape, 1024 rows: QKV 142 / 188, O 59 / 71,              gate/up 232 / 315, down 134 / 169
+//   13B shape, 1024 rows: QKV 223 / 272, O 119 / 123,           gate/up 352 / 471, down 308 / 312
+//   1B shape,  160 rows: QKV 32 / 22 / 25, 26,  O 34 / 23 / 26, 26, 28,  gate/up 32 / 38,  down 90 / 61 / 45, 40, 38
+// (a merge costs as much as 25 to 40 K blocks, so K of 2048 is not cut)
 struct Split { int bn, parts; double us; };
 Split choose_split(int epi, const Dims &D, int M, int n_sms) {
     const int K = epi == PF_OPROJ ? D.nh * D.hd : (epi == PF_DOWN ? D.F : D.d);
@@ -533,13 +536,19 @@ Split choose_split(int epi, const Dims &D, int M, int n_sms) {
         for (int parts = 1; parts <= (bn == 128 ? 4 : 1); ++parts) {
             const int tiles = n_mt * n_tiles_of(epi, D, bn) * parts;
             if (parts > 1 && (tiles > n_sms || tiles > DEL_WT_CTAS || n_kb < 4 * parts)) continue;
-            const double us = (tiles + n_sms - 1) / n_sms * ((double)n_kb / parts * (bn == 256 ? 0.70 : 0.45)) + (bn == 256 ? 8 : 4) + (parts > 1 ? 3 + parts : 0);
+            const double us = (tiles + n_sms - 1) / n_sms * ((double)n_kb / parts * (bn == 256 ? 0.667 : 0.452)) + (bn == 256 ? 12 : 8.3) + (parts > 1 ? 5 + 2.3 * parts : 0);
             if (best.bn == 0 || us < best.us) best = Split{bn, parts, us};
         }
     return best;
 }
 
 }  // namespace
+
+void prefill_tc_split(int epi, const Dims &D, int M, int n_sms, int *bn, int *parts) {
+    const Split s = choose_split(epi, D, M, n_sms);
+    *bn = s.bn;
+    *parts = s.parts;
+}
 
 // Positions per chunk of a prompt of n: the whole number of 128-row tiles, at most max_rows, with the smallest estimated
 // time of the four GEMMs over all chunks (a wave of tiles that is nearly empty costs as much as a full one: the 13B shape's
