@@ -385,15 +385,22 @@ CtlArgs ctl_base(const del_ctx *c, int plan_idx) {
 
 // Rows from which on a pass's layer GEMMs run on tcgen05 (rowgemm_tc.cu) rather than register streaming (rowgemm.cu).  The
 // former has a fixed cost of about 14 us per layer (four launches with a ticket and a merge at their end), the latter one
-// that grows with the rows and the weight bytes.  Measured, us per layer, register streaming / tcgen05:
-//   13B shape (635 MB)   5 rows 139 / 128,   8: 148 / 130,   13: 209 / 135
-//   8B shape (436 MB)    5 rows 104 / 107,   8: 107 / 107,    9: 138 / 110,   16: 155 / 114,   32: 268 / 140
-//   7B shape (405 MB)    5 rows  90 /  95,   8:  95 /  96,    9: 123 /  97,   16: 140 / 100,   32: 251 / 121
-//   1B shape (122 MB)    8 rows  50 /  63,   9:  65 /  67,   16:  74 /  68,   32: 112 /  92
-//   tiny (1.6 MB)        8 rows  18 /  34,  16:  24 /  34,   32:  33 /  47
+// that grows with the rows and the weight bytes (and doubles at 33 rows: two launches).  The lines lie where no measured pass
+// is more than 3 % slower than with register streaming.  us per layer, register streaming / tcgen05:
+//   13B shape (635 MB)   4 rows 126 / 131,   5: 138 / 131,   8: 148 / 132,   13: 219 / 137
+//   570 MB               4 rows 116 / 121,   5: 130 / 122,   8: 137 / 123,    9: 189 / 131
+//   510 MB               5 rows 105 / 111,   8: 115 / 113,   9: 149 / 117,   16: 171 / 118
+//   8B shape (436 MB)    5 rows  99 / 101,   8: 106 / 104,   9: 138 / 105,   16: 158 / 110,   32: 280 / 132
+//   7B shape (405 MB)    5 rows  89 /  95,   8:  93 /  98,   9: 126 / 102,   16: 141 / 102,   32: 258 / 124
+//   1B shape (122 MB)    8 rows  47 /  60,   9:  64 /  63,  16:  73 /  64,   32: 110 /  89
+//   88 MB                9 rows  59 /  61,  16:  69 /  65,  17:  86 /  82,   32: 105 /  92
+//   78 MB               16 rows  58 /  58,  17:  75 /  76,  32:  87 /  86,   33: 112 /  98
+//   67 MB               17 rows  75 /  82,  32:  94 / 100,  33: 118 / 112,   64: 186 / 172
+//   50 MB               32 rows  72 /  81,  33:  91 /  93,  48: 119 / 104,   64: 137 / 140
+//   tiny (1.6 MB)        8 rows  17 /  34,  16:  24 /  36,  32:  33 /  52
 int rows_min_tc(const Dims &D) {
     const double mb = 2e-6 * ((double)D.d * (D.nh + 2 * D.nkv) * D.hd + (double)D.nh * D.hd * D.d + 3.0 * D.d * D.F);
-    return mb >= 500 ? 5 : (mb >= 100 ? 9 : (mb >= 64 ? 17 : DEL_ROWS_MAX + 1));
+    return mb >= 550 ? 5 : mb >= 100 ? 9 : mb >= 80 ? 17 : mb >= 64 ? 33 : DEL_ROWS_MAX + 1;
 }
 
 struct PassInfo {

@@ -81,3 +81,32 @@ def test_prefill_tiles_are_near_the_best_measured(line):
     split = dl.debug_routes(dl.make_shape(CONFIGS[name]), SMS, int(rows), int(rows))[2][["qkv", "o", "gate_up", "down"].index(gemm)]
     us = dict(zip([(256, 1), (128, 1), (128, 2), (128, 3), (128, 4)], map(float, us)))
     assert us[split] <= 1.08 * min(us.values()), (split, us)
+
+
+# d_model, heads, kv heads, head dimension, d_ffn; then us per layer of a pass of so many rows: register streaming / tcgen05
+PASSES = """
+1536,24,8,64,4096        4:28/46 5:32/45 8:34/47 9:45/52 16:50/53 17:59/71 24:66/76 32:72/81 33:91/93 48:119/104 64:137/140
+1792,28,4,64,4864        4:32/51 5:37/51 8:39/53 9:52/59 16:62/63 17:75/82 24:83/87 32:94/100 33:118/112 48:157/129 64:186/172
+2048,32,8,64,4608        4:32/50 5:37/51 8:40/53 9:52/56 16:58/58 17:75/76 24:79/81 32:87/86 33:112/98 48:140/107 64:168/144
+2048,32,4,64,5632        4:34/53 5:40/53 8:43/55 9:59/61 16:69/65 17:86/82 24:93/84 32:105/93 33:133/109 48:171/122 64:208/165
+2048,32,8,64,8192        4:36/59 5:44/58 8:47/60 9:64/64 16:73/64 17:94/81 24:100/85 32:110/90 33:141/103 48:180/111 64:216/145
+4096,32,32,128,11008     4:83/96 5:89/95 8:93/98 9:126/102 16:141/102 17:224/116 24:236/118 32:258/124 33:327/137 48:393/141 64:508/162
+4096,32,8,128,14336      4:88/103 5:99/101 8:106/104 9:138/105 16:158/110 17:245/124 24:256/126 32:280/132 33:359/148 48:432/156 64:561/187
+4608,36,36,128,12288     4:99/111 5:105/111 8:115/113 9:149/117 16:171/118 17:244/132 24:262/134 32:285/139 33:372/152 48:450/155 64:564/173
+4864,38,38,128,13056     4:116/121 5:130/122 8:137/123 9:189/131 16:214/130 17:315/142 24:332/145 32:361/148 33:470/165 48:573/170 64:715/187
+5120,40,40,128,13824     4:126/131 5:140/132 8:148/132 9:205/138 16:234/139 17:329/154 24:348/155 32:378/161 33:493/176 48:606/179 64:746/201
+256,4,4,64,688           4:18/33 5:17/33 8:17/34 9:23/36 16:24/36 17:30/50 24:31/50 32:33/52 33:49/63 48:54/66 64:58/79
+"""
+
+
+@pytest.mark.parametrize("line", PASSES.strip().splitlines(), ids=lambda s: s.split()[0])
+def test_layer_passes_are_not_slower_than_register_streaming(line):
+    """3 %: the spread of a pass's time between runs."""
+    import paper_2504_05598_b200 as dl
+    shape, *rows = line.split()
+    d, nh, nkv, hd, F = map(int, shape.split(","))
+    cfg = synth.small_variant(TINY, d_model=d, n_heads=nh, n_kv_heads=nkv, head_dim=hd, d_ffn=F)
+    rows_min = dl.debug_routes(dl.make_shape(cfg), SMS, 1, 1)[0]
+    for r in rows:
+        n, (streaming, tc) = int(r.split(":")[0]), map(float, r.split(":")[1].split("/"))
+        assert n < rows_min or tc <= 1.03 * streaming, (rows_min, r)
