@@ -114,12 +114,15 @@ typedef struct {
     double next_tau;              /* Eq. 3 for layer next_E from the updated statistics */
 } del_round_out;
 
-/* Bytes of DEVICE workspace del_init needs for this shape (256-byte aligned base expected). */
+/* Bytes of DEVICE workspace for this shape (256-byte aligned base expected).  They include the buffers in which a prompt goes
+ * through the layers in chunks of up to 2048 positions (or max_seq, if that is less): 124 KB per position at the 7B shape, 155 KB
+ * at the 13B shape.  del_init also takes less, down to one tile of 128 positions: longer prompts then go in more and shorter
+ * chunks, with the same results but for the order of sums, and slower (a chunk streams the layers' weights once). */
 size_t del_workspace_bytes(const del_shape *shape);
 
-/* Creates a context.  shape, weights, kv: HOST structs (copied).  workspace: DEVICE, ws_bytes >=
- * del_workspace_bytes(shape); its contents are clobbered.  cuda_stream: a cudaStream_t (0 = default
- * stream).  Errors: DEL_EINVAL (shape requirements, null pointers), DEL_ENOSPC (workspace too small,
+/* Creates a context.  shape, weights, kv: HOST structs (copied).  workspace: DEVICE, ws_bytes =
+ * del_workspace_bytes(shape), or less as said there; its contents are clobbered.  cuda_stream: a cudaStream_t (0 = default
+ * stream).  Errors: DEL_EINVAL (shape requirements, null pointers), DEL_ENOSPC (workspace too small for a 128-position chunk,
  * n_pages cannot hold even one sequence), DEL_ECUDA. */
 int del_init(del_ctx **ctx, const del_shape *shape, const del_weights *weights, const del_kv *kv,
              void *workspace, size_t ws_bytes, void *cuda_stream);

@@ -185,9 +185,10 @@ class DelContext:
 
     ``weights``: dict with bf16 CUDA tensors ``tok_emb``, ``final_norm``, ``lm_head`` and a list ``layers`` of
     dicts with ``attn_norm, wq, wk, wv, wo, ffn_norm, w_gate, w_up, w_down`` (matrices [out, in]).
+    ``workspace_bytes``: less device memory than ``del_workspace_bytes`` asks for (long prompts then run in shorter chunks).
     """
 
-    def __init__(self, shape: Shape, weights: Dict, device="cuda:0", stream=None):
+    def __init__(self, shape: Shape, weights: Dict, device="cuda:0", stream=None, workspace_bytes: Optional[int] = None):
         import torch
         if not torch.cuda.is_available():
             raise RuntimeError("libdel needs a CUDA device; there is no CPU fallback")
@@ -210,6 +211,8 @@ class DelContext:
             ws = self.lib.del_workspace_bytes(C.byref(shape))
             if ws == 0:
                 raise DelError(EINVAL, "del_workspace_bytes")
+            if workspace_bytes is not None:
+                ws = min(ws, workspace_bytes)
             self.workspace = torch.empty(ws + 256, dtype=torch.uint8, device=self.device)
             ws_ptr = (self.workspace.data_ptr() + 255) // 256 * 256
             wc = WeightsC()

@@ -84,6 +84,7 @@ struct del_ctx {
     bool wt_ok = false;
     int wt_rows_min = DEL_ROWS_MAX + 1;                   // rows from which on a pass takes that form
     bool pf_ok = false;
+    int pf_rows = 0;                                      // positions the chunk buffers hold
     // mailbox of the draft loop's confidence check: pinned host memory that the finalise kernel writes directly
     volatile float *post_conf = nullptr;
     volatile uint32_t *post_stamp = nullptr;
@@ -109,10 +110,11 @@ struct del_ctx {
 
 namespace {
 
-// rows of the bulk prefill's chunk buffers: a chunk, or all a sequence can hold (whole 128-row tiles)
+// rows of the bulk prefill's chunk buffers in a workspace of del_workspace_bytes: a chunk, or all a sequence can hold (whole
+// 128-row tiles)
 int prefill_rows(const del_shape &s) { return std::min(PF_ROWS, (s.max_seq + 127) / 128 * 128); }
 
-size_t carve_all(const del_shape &s, void *base, Dims &D, Buffers &B, int &R_max, int &n_vtiles,
+size_t carve_all(const del_shape &s, int pf_rows, void *base, Dims &D, Buffers &B, int &R_max, int &n_vtiles,
                  del_round_out **out_dev, float **dbg_dev, PfArgs *pf, WtBuffers *wt) {
     D.L = s.n_layers; D.d = s.d_model; D.nh = s.n_heads; D.nkv = s.n_kv_heads; D.hd = s.head_dim; D.F = s.d_ffn; D.V = s.vocab;
     D.B = s.max_batch;
@@ -173,8 +175,7 @@ size_t carve_all(const del_shape &s, void *base, Dims &D, Buffers &B, int &R_max
     *out_dev = c.take<del_round_out>(base, (size_t)D.B);
     B.ERR = c.take<int32_t>(base, 64);           // right behind the results: one copy brings both to the host
     *dbg_dev = c.take<float>(base, (size_t)std::max(D.V, 2 * D.nkv * D.hd));
-    // chunk buffers of the bulk prefill (PF_ROWS prompt positions)
-    const int pf_rows = prefill_rows(s);
+    // chunk buffers of the bulk prefill (pf_rows prompt positions)
     PfArgs pfa;
     memset(&pfa, 0, sizeof(pfa));
     pfa.n_ssp = prefill_tc_nssp(D);
@@ -196,10 +197,22 @@ size_t carve_all(const del_shape &s, void *base, Dims &D, Buffers &B, int &R_max
     wtb.n_tickets = std::max({DEL_WT_CTAS, rowgemm_tc_tiles(EPI_QKV, D), rowgemm_tc_tiles(EPI_GATEUP, D), rowgemm_tc_tiles(EPI_DOWN, D)});
     wtb.xd = c.take<bf16>(base, (size_t)DEL_ROWS_MAX * D.d);
     wtb.xdl = c.take<bf16>(base, (size_t)DEL_ROWS_MAX * D.d);
-    wtb.part = c.take<float>(base, (size_t)DEL_WT_CTAS * 2 * DEL_ROWS_MAX * 128);
+    wtb.part = c.take<float>(base, (size_t)rowgemm_tc_ctas(D) * 2 * DEL_ROWS_MAX * 128);
     wtb.ticket = c.take<int32_t>(base, (size_t)wtb.n_tickets);
     if (wt) *wt = wtb;
     return (c.off + 255) & ~(size_t)255;
+}
+
+size_t workspace_bytes(const del_shape &s, int pf_rows) {
+    Dims D; Buffers B; int R, nv; del_round_out *o; float *dbg;
+    return carve_all(s, pf_rows, nullptr, D, B, R, nv, &o, &dbg, nullptr, nullptr);
+}
+
+// the most chunk rows that fit into ws_bytes; 0: not even one tile of them
+int prefill_rows_in(const del_shape &s, size_t ws_bytes) {
+    int rows = prefill_rows(s);
+    while (rows > 0 && workspace_bytes(s, rows) > ws_bytes) rows -= 128;
+    return rows;
 }
 
 int validate(const del_shape *s) {
@@ -736,7 +749,7 @@ int draft_with_exit(del_ctx *c, std::vector<Job> &jobs) {
 int prefill_bulk(del_ctx *c, int sq, int n_pos, int win0) {
     const Dims &D = c->D;
     const bool P = pdl(c);
-    const int chunk = prefill_tc_chunk(D, n_pos, c->n_sms, prefill_rows(c->sh));
+    const int chunk = prefill_tc_chunk(D, n_pos, c->n_sms, c->pf_rows);
     for (int p0 = 0; p0 < n_pos; p0 += chunk) {
         PfArgs a = c->pf;
         a.M = std::min(chunk, n_pos - p0);
@@ -1046,14 +1059,13 @@ extern "C" {
 
 size_t del_workspace_bytes(const del_shape *shape) {
     if (validate(shape) != DEL_OK) return 0;
-    Dims D; Buffers B; int R, nv; del_round_out *o; float *dbg;
-    return carve_all(*shape, nullptr, D, B, R, nv, &o, &dbg, nullptr, nullptr);
+    return workspace_bytes(*shape, prefill_rows(*shape));
 }
 
 int del_debug_routes(const del_shape *shape, int n_sms, int n_prompt, int rows, int32_t *out) {
     if (validate(shape) != DEL_OK || n_sms < 1 || n_prompt < 1 || rows < 1 || !out) return DEL_EINVAL;
     Dims D; Buffers B; int R, nv; del_round_out *o; float *dbg;
-    carve_all(*shape, nullptr, D, B, R, nv, &o, &dbg, nullptr, nullptr);
+    carve_all(*shape, prefill_rows(*shape), nullptr, D, B, R, nv, &o, &dbg, nullptr, nullptr);
     out[0] = rowgemm_tc_supported(D) ? rows_min_tc(D) : DEL_ROWS_MAX + 1;
     out[1] = prefill_tc_chunk(D, n_prompt, n_sms, prefill_rows(*shape));
     for (int epi = PF_QKV; epi <= PF_DOWN; ++epi) {
@@ -1074,11 +1086,13 @@ int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const 
         !w->ffn_norm || !w->w_gate || !w->w_up || !w->w_down || !w->rope_cos || !w->rope_sin)
         return DEL_EINVAL;
     if (!kv->k_pages || !kv->v_pages || !kv->page_table) return DEL_EINVAL;
-    if (ws_bytes < del_workspace_bytes(shape)) return DEL_ENOSPC;
+    const int pf_rows = prefill_rows_in(*shape, ws_bytes);
+    if (pf_rows == 0) return DEL_ENOSPC;
     del_ctx *c = new (std::nothrow) del_ctx();
     if (!c) return DEL_ENOSPC;
     c->sh = *shape;
-    carve_all(*shape, workspace, c->D, c->B, c->R_max, c->n_vtiles, &c->out_dev, &c->dbg_dev, &c->pf, &c->wt);
+    c->pf_rows = pf_rows;
+    carve_all(*shape, pf_rows, workspace, c->D, c->B, c->R_max, c->n_vtiles, &c->out_dev, &c->dbg_dev, &c->pf, &c->wt);
     c->B.KP = (bf16 *)kv->k_pages; c->B.VP = (bf16 *)kv->v_pages; c->B.PT = kv->page_table;
     c->B.rope_cos = w->rope_cos; c->B.rope_sin = w->rope_sin;
     c->tok_emb = (const bf16 *)w->tok_emb; c->final_norm = (const bf16 *)w->final_norm; c->lm_head = (const bf16 *)w->lm_head;
@@ -1126,7 +1140,7 @@ int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const 
         }
     }
     // zero the workspace (counters, statistics) and the KV pages (stale bit patterns must stay finite)
-    if (e == cudaSuccess) e = cudaMemsetAsync(workspace, 0, del_workspace_bytes(shape), c->st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(workspace, 0, workspace_bytes(*shape, pf_rows), c->st);
     const size_t kv_bytes = (size_t)shape->n_pages * L * shape->n_kv_heads * 16 * shape->head_dim * sizeof(bf16);
     if (e == cudaSuccess) e = cudaMemsetAsync(kv->k_pages, 0, kv_bytes, c->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(kv->v_pages, 0, kv_bytes, c->st);
@@ -1140,7 +1154,6 @@ int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const 
                lmhead_tc_make_map(c->map_w, c->lm_head, (uint64_t)shape->vocab, (uint64_t)shape->d_model, 256) == 0;
     {
         // tensor maps of the bulk prefill and of the weights: boxes of 128 rows (gate / up: 64)
-        const uint64_t pf_rows = prefill_rows(*shape);
         const uint64_t d = shape->d_model, qd = (uint64_t)shape->n_heads * shape->head_dim,
                        kvd = (uint64_t)shape->n_kv_heads * shape->head_dim, F = shape->d_ffn;
         bool ok = lmhead_tc_make_map(c->pf_xs.b, c->pf.XS, pf_rows, d, 128) == 0 &&

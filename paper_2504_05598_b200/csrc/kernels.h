@@ -49,11 +49,12 @@ int rowgemm_lmhead_grid(int n_items, int m, int n_sms, int ctas_per_sm);
 #define DEL_WT_CTAS 160        // most CTAs of such a launch (partial sums in the workspace: 2 x 128 x 64 floats each)
 struct WtBuffers {
     bf16 *xd, *xdl;            // [ROWS][d] the next layer's input by row of the pass, written by DOWN beside the hidden stack
-    float *part;               // partial sums of tiles that several CTAs share
+    float *part;               // partial sums of tiles that several CTAs share (room for rowgemm_tc_ctas CTAs)
     int32_t *ticket;           // [tiles] arrivals at such a tile; zero between launches
     int32_t n_tickets;
 };
 int rowgemm_tc_tiles(int epi, const Dims &D);
+int rowgemm_tc_ctas(const Dims &D);                    // most CTAs of a launch of this shape (at most DEL_WT_CTAS)
 bool rowgemm_tc_supported(const Dims &D);
 bool rowgemm_tc_fits(const GemmArgs &a);               // whether a QKV launch can read the pass's rows from the hidden stack
 cudaError_t launch_rowgemm_tc(int epi, const GemmArgs &a, const void *map_w0, const void *map_w1, const void *map_w2, const void *map_x,

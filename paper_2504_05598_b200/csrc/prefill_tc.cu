@@ -535,7 +535,7 @@ Split choose_split(int epi, const Dims &D, int M, int n_sms) {
     for (int bn = 256; bn >= 128; bn -= 128)
         for (int parts = 1; parts <= (bn == 128 ? 4 : 1); ++parts) {
             const int tiles = n_mt * n_tiles_of(epi, D, bn) * parts;
-            if (parts > 1 && (tiles > n_sms || tiles > DEL_WT_CTAS || n_kb < 4 * parts)) continue;
+            if (parts > 1 && (tiles > n_sms || tiles > rowgemm_tc_ctas(D) || n_kb < 4 * parts)) continue;
             const double us = (tiles + n_sms - 1) / n_sms * ((double)n_kb / parts * (bn == 256 ? 0.667 : 0.452)) + (bn == 256 ? 12 : 8.3) + (parts > 1 ? 5 + 2.3 * parts : 0);
             if (best.bn == 0 || us < best.us) best = Split{bn, parts, us};
         }

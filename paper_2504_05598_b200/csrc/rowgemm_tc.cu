@@ -532,6 +532,15 @@ int rowgemm_tc_tiles(int epi, const Dims &D) {
     }
 }
 
+int rowgemm_tc_ctas(const Dims &D) {
+    int most = 0;
+    for (int epi = EPI_QKV; epi <= EPI_DOWN; ++epi) {
+        const int K = epi == EPI_OPROJ ? D.nh * D.hd : (epi == EPI_DOWN ? D.F : D.d);
+        most = max(most, min(DEL_WT_CTAS, rowgemm_tc_tiles(epi, D) * ((K + BK - 1) / BK)));
+    }
+    return most;
+}
+
 bool rowgemm_tc_supported(const Dims &D) {
     const int k = D.F > D.nh * D.hd ? D.F : D.nh * D.hd, kmax = k > D.d ? k : D.d;
     const long long tiles = rowgemm_tc_tiles(EPI_QKV, D) > rowgemm_tc_tiles(EPI_GATEUP, D) ? rowgemm_tc_tiles(EPI_QKV, D) : rowgemm_tc_tiles(EPI_GATEUP, D);
