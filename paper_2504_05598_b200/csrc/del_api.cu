@@ -1188,6 +1188,11 @@ int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const 
                    lmhead_tc_make_map(c->wt_xml.b, c->B.XML, DEL_ROWS_MAX, d, 16) == 0 &&
                    lmhead_tc_make_map(c->wt_act.b, c->B.ACT, DEL_ROWS_MAX, F, 16) == 0 &&
                    lmhead_tc_make_map(c->wt_actl.b, c->B.ACTL, DEL_ROWS_MAX, F, 16) == 0;
+        if ((c->pf_ok && prefill_tc_prepare() != cudaSuccess) ||
+            (c->wt_ok && c->wt_rows_min <= DEL_ROWS_MAX && rowgemm_tc_prepare() != cudaSuccess)) {
+            del_destroy(c);
+            return DEL_ECUDA;
+        }
         c->pfa_ok = ok && prefill_attention_tc_supported(c->D) &&
                     lmhead_tc_make_map(c->pf_q.b, c->pf.Q, pf_rows, qd, 128) == 0 &&
                     lmhead_tc_make_map(c->pf_ql.b, c->pf.QL, pf_rows, qd, 128) == 0 &&

@@ -57,6 +57,9 @@ int rowgemm_tc_tiles(int epi, const Dims &D);
 int rowgemm_tc_ctas(const Dims &D);                    // most CTAs of a launch of this shape (at most DEL_WT_CTAS)
 bool rowgemm_tc_supported(const Dims &D);
 bool rowgemm_tc_fits(const GemmArgs &a);               // whether a QKV launch can read the pass's rows from the hidden stack
+// Loads the kernels onto the current device.  Left to the first launch of each, that costs 2 to 4 ms in the first round or prompt
+// of a process that carries 9 rows and more, and 0.3 to 1 ms in the first of 17, 33 and 49.
+cudaError_t rowgemm_tc_prepare();
 cudaError_t launch_rowgemm_tc(int epi, const GemmArgs &a, const void *map_w0, const void *map_w1, const void *map_w2, const void *map_x,
                               const void *map_xl, bool dense, const WtBuffers &b, int n_sms, cudaStream_t st, bool pdl);
 
@@ -207,6 +210,7 @@ struct PfArgs {
     float *stackH;
     int32_t win0;
 };
+cudaError_t prefill_tc_prepare();              // loads the kernels onto the current device (rowgemm_tc_prepare)
 int prefill_tc_chunk(const Dims &D, int n, int n_sms, int max_rows);
 void prefill_tc_split(int epi, const Dims &D, int M, int n_sms, int *bn, int *parts);      // what launch_prefill_gemm chooses
 int prefill_tc_nssp(const Dims &D);            // partial sums of squares per row

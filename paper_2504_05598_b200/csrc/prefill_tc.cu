@@ -26,6 +26,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <initializer_list>
 
 #include "kernels.h"
 #include "tc_common.cuh"
@@ -479,20 +480,25 @@ __global__ void __launch_bounds__(256) prefill_embed_kernel(const PfArgs p, cons
     }
 }
 
+constexpr size_t SMEM_BYTES = (size_t)RING_BYTES + 1024;
+
+template <int EPI> cudaError_t prepare_epi() {
+    static SmemAttrOnce attr;
+    return attr.set(prefill_gemm_kernel<EPI>, (int)SMEM_BYTES);
+}
+
 template <int EPI>
 cudaError_t launch_epi(const PfMaps &maps, const PfArgs &p, int n_sms, cudaStream_t st, bool pdl) {
-    const size_t smem = (size_t)RING_BYTES + 1024;
     auto kern = prefill_gemm_kernel<EPI>;
-    static SmemAttrOnce attr;
     {
-        cudaError_t e = attr.set(kern, (int)((int)smem));
+        cudaError_t e = prepare_epi<EPI>();
         if (e != cudaSuccess) return e;
     }
     const int n_tiles = ((p.M + BM - 1) / BM) * p.n_ntiles * p.k_parts;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_tiles < n_sms ? n_tiles : n_sms);
     cfg.blockDim = dim3(PF_THREADS);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -566,6 +572,13 @@ int prefill_tc_chunk(const Dims &D, int n, int n_sms, int max_rows) {
         if (best == 0 || us < best_us) { best = c; best_us = us; }
     }
     return best;
+}
+
+cudaError_t prefill_tc_prepare() {
+    for (cudaError_t e : {prepare_epi<PF_QKV>(), prepare_epi<PF_OPROJ>(), prepare_epi<PF_GATEUP>(), prepare_epi<PF_DOWN>()})
+        if (e != cudaSuccess) return e;
+    cudaFuncAttributes a;
+    return cudaFuncGetAttributes(&a, prefill_embed_kernel);
 }
 
 // map_a / map_b*: 128-byte CUtensorMap blobs made by lmhead_tc_make_map (boxes of 128 rows, W_gate / W_up 64)

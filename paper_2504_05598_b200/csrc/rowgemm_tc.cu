@@ -26,6 +26,7 @@
 #include <cuda.h>
 
 #include <cstring>
+#include <initializer_list>
 
 #include "kernels.h"
 #include "tc_common.cuh"
@@ -473,13 +474,25 @@ __global__ void __launch_bounds__(WT_THREADS, 1) rowgemm_tc_kernel(const __grid_
     if (threadIdx.x == 0 && s_err) atomicMax(a.B.ERR, (int)s_err);
 }
 
+template <int NP> constexpr size_t smem_bytes() { return (size_t)stages<NP>() * (W_BYTES + x_bytes<NP>()) + 1024; }
+
+template <int NP, int EPI> cudaError_t prepare_np() {
+    static SmemAttrOnce attr;
+    return attr.set(rowgemm_tc_kernel<NP, EPI>, (int)smem_bytes<NP>());
+}
+
+template <int NP> cudaError_t prepare_rows() {
+    for (cudaError_t e : {prepare_np<NP, EPI_QKV>(), prepare_np<NP, EPI_OPROJ>(), prepare_np<NP, EPI_GATEUP>(), prepare_np<NP, EPI_DOWN>()})
+        if (e != cudaSuccess) return e;
+    return cudaSuccess;
+}
+
 template <int NP, int EPI>
 cudaError_t launch_np(const WtMaps &maps, const WtArgs &w, int n_sms, cudaStream_t st, bool pdl) {
-    const size_t smem = (size_t)stages<NP>() * (W_BYTES + x_bytes<NP>()) + 1024;
+    const size_t smem = smem_bytes<NP>();
     auto kern = rowgemm_tc_kernel<NP, EPI>;
-    static SmemAttrOnce attr;
     {
-        cudaError_t e = attr.set(kern, (int)smem);
+        cudaError_t e = prepare_np<NP, EPI>();
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
@@ -546,6 +559,12 @@ bool rowgemm_tc_supported(const Dims &D) {
     const long long tiles = rowgemm_tc_tiles(EPI_QKV, D) > rowgemm_tc_tiles(EPI_GATEUP, D) ? rowgemm_tc_tiles(EPI_QKV, D) : rowgemm_tc_tiles(EPI_GATEUP, D);
     const long long rows = tiles > rowgemm_tc_tiles(EPI_DOWN, D) ? tiles : rowgemm_tc_tiles(EPI_DOWN, D);
     return (rows * ((kmax + BK - 1) / BK) + 1) * DEL_WT_CTAS < (1ll << 31);
+}
+
+cudaError_t rowgemm_tc_prepare() {
+    for (cudaError_t e : {prepare_rows<16>(), prepare_rows<32>(), prepare_rows<48>(), prepare_rows<64>()})
+        if (e != cudaSuccess) return e;
+    return cudaSuccess;
 }
 
 bool rowgemm_tc_fits(const GemmArgs &a) {

@@ -80,3 +80,44 @@ def test_prompt_kernels_against_decode_kernels(cfg, prompt_len):
     for a, b in zip(*got):
         assert np.linalg.norm(a - b) <= 2.0 ** -7 * np.linalg.norm(b)
     ctx.close()
+
+
+FIRST_PASS = """
+import time
+import numpy as np, torch
+import paper_2504_05598_b200 as dl, synth
+cfg = synth.small_variant(synth.CONFIGS["tiny"], n_layers=2, d_model=2048, n_heads=32, n_kv_heads=8, head_dim=64, d_ffn=8192,
+                          prompt_len=64, e_max=1, init_window=1)
+dims = dict(attn_norm=(2048,), wq=(2048, 2048), wk=(512, 2048), wv=(512, 2048), wo=(2048, 2048), ffn_norm=(2048,),
+            w_gate=(8192, 2048), w_up=(8192, 2048), w_down=(2048, 8192))
+new = lambda *s: torch.randn(s, device="cuda", dtype=torch.bfloat16) * 0.02
+w = dict(tok_emb=new(1024, 2048), final_norm=new(2048), lm_head=new(1024, 2048),
+         layers=[{k: new(*s) for k, s in dims.items()} for _ in range(2)])
+assert dl.debug_routes(dl.make_shape(cfg), 148, 1, 1)[0] <= 16
+ctx = dl.DelContext(dl.make_shape(cfg), w)
+p = np.arange(64, dtype=np.int32)
+def t(n):
+    t0 = time.perf_counter(); ctx.prefill(0, p[:n], 2); return time.perf_counter() - t0
+t(2); t(2)                                    # everything but the layer GEMMs of 16 rows
+for n in (17, 48):                            # a pass of 16 rows, and a prompt for the prefill kernels
+    first, again = t(n), min(t(n), t(n))
+    print(first / again)
+"""
+
+
+def test_first_pass_of_many_rows_loads_no_code():
+    """del_init loads the tcgen05 layer and prefill GEMMs: the first pass that takes them is no slower than the next (loading
+    takes the time of 3 to 10 of these; what is left is the prefill attention kernel).
+    Another process on the machine can hold up one run, hence three tries."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    seen = []
+    for _ in range(3):
+        r = subprocess.run([sys.executable, "-c", FIRST_PASS], cwd=root, capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
+        seen.append([float(x) for x in r.stdout.split()])
+        if max(seen[-1]) < 3:
+            return
+    assert False, seen
