@@ -265,10 +265,10 @@ int del_get_hidden(del_ctx *ctx, int seq, int layer, int row, float *out);
 int del_debug_logits(del_ctx *ctx, int seq, int layer, int row, float *out);
 int del_get_kv(del_ctx *ctx, int seq, int layer, int pos, float *k_out, float *v_out);
 
-/* DEL_ETIMEOUT.  The tensor-core kernels (stacked LM head, prefill GEMMs) wait on shared-memory barriers for
+/* DEL_ETIMEOUT.  The tensor-core kernels (stacked LM head, layer GEMMs of many rows, prefill) wait on shared-memory barriers for
  * their own asynchronous copies and tensor-core instructions.  Every such wait gives up after 2^26 polls
  * (of the order of seconds to a minute, depending on the clock), records a non-zero code in the workspace's
- * error word, lets the kernel wind down (tensor memory freed) and return.  The call that next reads results
+ * error word, lets the kernel wind down (copies and MMAs in flight awaited, tensor memory freed) and return.  The call that next reads results
  * (del_prefill, del_layer_accept, del_select, del_round) then returns DEL_ETIMEOUT, clears the word, and the
  * context stays usable: the sequence's round did not complete and should be re-prefilled.
  * del_debug_inject_error writes `code` (non-zero) into that word with a stream-ordered copy from the host, as

@@ -92,6 +92,7 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                     tma_load_2d(sa + A_BYTES, &map_w, kb * BK, vt * BN, &full_bar[s]);
                 }
             }
+            if (s_err) drain(full_bar, STAGES, it % STAGES, (uint32_t)(it / STAGES) & 1);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -118,6 +119,7 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 if (!ok) break;
                 umma_commit(&tfull_bar[buf]);        // accumulator complete
             }
+            if (s_err) drain(empty_bar, STAGES, it % STAGES, (uint32_t)(it / STAGES) & 1);
         }
     } else {
         const int q = warp & 3;                      // TMEM lane quarter this warp may read

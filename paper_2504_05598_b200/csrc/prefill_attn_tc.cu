@@ -135,7 +135,8 @@ __global__ void __launch_bounds__(THREADS, 1) prefill_attention_tc_kernel(const 
         const int32_t *pt = p.PT + p.seq * p.D.pages_per_seq;
         auto page_of = [&](int pi) { return pi < p.D.pages_per_seq && pi < 4 * n_kb ? pt[pi] : 0; };   // (pages past the sequence: any page, masked)
         int cur = page_of(lane), nxt = page_of(32 + lane);
-        for (int j = 0; j < n_kb; ++j) {
+        int j = 0;
+        for (; j < n_kb; ++j) {
             const int s = j % KV_STAGES, first = (4 * j) & 31;
             if (first == 0 && j > 0) { cur = nxt; nxt = page_of(4 * j + 32 + lane); }
             int pages[4];
@@ -159,12 +160,17 @@ __global__ void __launch_bounds__(THREADS, 1) prefill_attention_tc_kernel(const 
             }
             if (!__shfl_sync(0xffffffffu, (int)ok, 0)) break;
         }
+        if (s_err && lane == 0) {
+            drain(&q_full, 1, 1, 0);
+            drain(kv_full, KV_STAGES, j % KV_STAGES, (uint32_t)(j / KV_STAGES) & 1);
+        }
     } else if (warp == 1) {
         if (lane == 0) {
             // instruction descriptors: fp32 accumulate, bf16 x bf16, both operands K-major, M = 128, N = 64 / 128
             const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BKEY >> 3) << 17) | ((uint32_t)(BQ >> 4) << 24);
             const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(HD >> 3) << 17) | ((uint32_t)(BQ >> 4) << 24);
             const uint32_t q_addr = smem_u32(q_sm), p_addr = smem_u32(p_sm);
+            int n_s = 0, n_o = 0;                    // blocks whose scores, whose products with the values have been issued
             bool ok = wait_or_err(&q_full, 0, &s_err);
             if (!ok && !s_err) s_err = 2;
             auto issue_scores = [&](int j) -> bool {
@@ -183,6 +189,7 @@ __global__ void __launch_bounds__(THREADS, 1) prefill_attention_tc_kernel(const 
                         for (int k = 0; k < 4; ++k) umma_bf16(d_tmem, da + 2 * k, db + 2 * k, idesc_s, (part | kb | k) != 0);
                     }
                 umma_commit(&s_full[buf]);
+                n_s = j + 1;
                 return true;
             };
             if (ok) ok = issue_scores(0);
@@ -202,6 +209,11 @@ __global__ void __launch_bounds__(THREADS, 1) prefill_attention_tc_kernel(const 
                 }
                 umma_commit(&kv_empty[s]);       // the stage's keys and values have been read
                 umma_commit(&o_done);            // the output holds blocks 0..j; the probabilities may be overwritten
+                n_o = j + 1;
+            }
+            if (s_err) {
+                drain(s_full, 2, n_s & 1, (uint32_t)(n_s >> 1) & 1);
+                drain(kv_empty, KV_STAGES, n_o % KV_STAGES, (uint32_t)(n_o / KV_STAGES) & 1);
             }
         }
     } else {

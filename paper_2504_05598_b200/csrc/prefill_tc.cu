@@ -366,6 +366,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
                     if (++s == n_stages) { s = 0; phase ^= 1; }
                 }
             }
+            if (s_err) drain(full_bar, n_stages, s, phase ^ 1);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -395,6 +396,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
                 if (!ok) break;
                 umma_commit(&tfull_bar[buf]);        // accumulator complete
             }
+            if (s_err) drain(empty_bar, n_stages, s, phase);
         }
     } else {
         const int q = warp & 3, half_id = (warp - 2) >> 2;   // TMEM lane quarter this warp may read, half of the columns

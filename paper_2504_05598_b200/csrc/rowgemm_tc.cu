@@ -294,6 +294,7 @@ __global__ void __launch_bounds__(WT_THREADS, 1) rowgemm_tc_kernel(const __grid_
                 }
                 if (++kb == nkb) { kb = 0; ++tile; }
             }
+            if (s_err) drain(full, STAGES, r.s, r.phase);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -323,6 +324,7 @@ __global__ void __launch_bounds__(WT_THREADS, 1) rowgemm_tc_kernel(const __grid_
                 umma_commit(&tfull[buf]);
                 u += n;
             }
+            if (s_err) drain(empty, STAGES, r.s, r.phase);
         }
     } else if (warp == 2) {
         if (lane == 0) {
@@ -354,6 +356,7 @@ __global__ void __launch_bounds__(WT_THREADS, 1) rowgemm_tc_kernel(const __grid_
                 }
                 if (++kb == nkb) kb = 0;
             }
+            if (s_err) drain(full, STAGES, r.s, r.phase);
         }
     } else if (warp >= 4) {
         const int q = warp & 3, half = (warp - 4) >> 2, et = threadIdx.x - 128, rr = q * 32 + lane;

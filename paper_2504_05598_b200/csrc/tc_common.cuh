@@ -32,6 +32,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity) {
         if (mbar_try(b, parity)) return true;
     return false;
 }
+// When a kernel gives up: waits, again bounded, for what this thread has started on a ring of n barriers, so that no copy lands
+// in shared memory and no MMA reads it once the CTA has left.  (s, phase): the stage that would come next and the parity of its
+// barrier's current phase.  (Whoever has left its loop before a wait gave up started its work 2^26 polls earlier.)
+__device__ __forceinline__ void drain(uint64_t *bars, int n, int s, uint32_t phase) {
+#pragma unroll 1
+    for (int i = 0; i < n; ++i)
+#pragma unroll 1
+        for (uint32_t t = 0; t < (1u << 18) && !mbar_try(&bars[i], i < s ? phase : phase ^ 1u); ++t) {}
+}
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
