@@ -745,7 +745,7 @@ int draft_with_exit(del_ctx *c, std::vector<Job> &jobs) {
 
 // ---- a whole prompt (positions 0 .. n_pos-1 of sequence sq) through the tensor-core GEMMs: the KV cache of
 // every position, and every layer's hidden state of the positions from win0 on (the window that seeds the
-// statistics) into the hidden stack; chunks of at most PF_ROWS positions, attention in passes of DEL_ROWS_MAX query rows
+// statistics) into the hidden stack; in chunks of at most as many positions as the chunk buffers hold
 int prefill_bulk(del_ctx *c, int sq, int n_pos, int win0) {
     const Dims &D = c->D;
     const bool P = pdl(c);

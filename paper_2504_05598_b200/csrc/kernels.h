@@ -178,7 +178,7 @@ cudaError_t launch_lmhead_tc(const void *map_x, const void *map_w, float *part_v
                              int n_sms, cudaStream_t st, bool pdl);
 
 // Prompt prefill on tcgen05 (prefill_tc.cu): tiled GEMMs over up to PF_ROWS prompt positions of one sequence
-// with the layer's element-wise work fused into the epilogues.  All buffers hold PF_ROWS rows (fewer if max_seq is smaller).
+// with the layer's element-wise work fused into the epilogues.  All buffers hold PF_ROWS rows (fewer if max_seq or the workspace is smaller).
 // prefill_tc_chunk picks the rows of a chunk up to this.  More rows leave less of a launch's last wave of tiles idle (7B
 // shape, 1000 positions: gate/up 5 waves in one chunk, 3 + 3 in two of 512, QKV 3 and 2 + 2: 679 and 860 us per layer); with
 // 2048 the widest activations (113 MB for the 13B shape's down projection) still about fit L2.

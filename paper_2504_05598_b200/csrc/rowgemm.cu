@@ -13,7 +13,8 @@
 // other's bursts, and the first burst of weights is issued before the kernel waits for its producer
 // (programmatic dependent launch).
 // Partial sums of the 8 warps are added in a fixed order through shared memory: results do not depend
-// on the grid size or on how many rows share the pass.
+// on the grid size or on how many rows share the launch.  (Passes with many rows run the layer GEMMs of rowgemm_tc.cu, which
+// add along K in another order: a row's last bits depend on which of the two its pass takes.)
 //
 // Activation precision.  The layer GEMMs take every activation as a pair of bf16 values (high + low part, 16
 // bits of mantissa; the weights are exact bf16 anyway), so that the product carries fp32-like accuracy.  The

@@ -13,7 +13,7 @@
 // the same number of bytes whatever the number of tiles (the 32 tiles of a d x d projection would otherwise leave 116
 // of 148 SMs idle).  A tile cut by a range boundary is finished by whichever of its CTAs arrives last: each leaves its
 // partial sums in the workspace, takes a ticket, and the last one adds all parts in K order.  Results depend
-// neither on timing nor on the number of rows; nobody waits for another CTA.
+// neither on timing nor on the number of rows of such a pass; nobody waits for another CTA.
 //
 // Roles (384 threads): warp 0 streams weight blocks with TMA (the ring is filled before the kernel waits for its
 // producer: weights depend on nobody), warp 2 the activation rows (for QKV they lie scattered over the hidden stack:

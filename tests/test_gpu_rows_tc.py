@@ -13,11 +13,35 @@ RAGGED = synth.small_variant(TINY, name="ragged", d_model=288, n_heads=5, n_kv_h
                              gain_spread=0.1, init_window=32, seed=31)
 HD128 = synth.small_variant(TINY, name="hd128", d_model=512, n_heads=6, n_kv_heads=3, head_dim=128, d_ffn=1040, emb_scale=10.0,
                             gain_spread=0.1, init_window=32, seed=32)
+# many units per CTA: gate/up 385 tiles of 3 K blocks, QKV 256 tiles of 3, O 3 tiles of 128, down 3 tiles of 193
+MANY_UNITS = synth.small_variant(TINY, name="many_units", n_layers=2, e_max=1, d_model=288, n_heads=128, n_kv_heads=64, head_dim=128,
+                                 d_ffn=24592, emb_scale=10.0, gain_spread=0.1, init_window=1, seed=33)
 
 
 def make_ctx(cfg, w, **kw):
     import paper_2504_05598_b200 as dl
     return dl.DelContext(dl.make_shape(cfg, **kw), dl.upload_weights(w))
+
+
+def tc_units(cfg):
+    """(tiles, K blocks per tile) of the tcgen05 launches QKV, O, gate/up, down."""
+    up = lambda n, k: -(-n // k)  # noqa: E731
+    d, q, kv, F = cfg.d_model, cfg.n_heads * cfg.head_dim, cfg.n_kv_heads * cfg.head_dim, cfg.d_ffn
+    return [(up(q, 128) + 2 * up(kv, 128), up(d, 128)), (up(d, 128), up(q, 128)), (up(F, 64), up(d, 128)), (up(d, 128), up(F, 128))]
+
+
+@pytest.mark.parametrize("rows", [9, 16, 17, 32, 33, 48, 49, 64])
+def test_forms_agree_with_many_units_per_cta(rows):
+    """The same where a CTA's range holds several units: the ring wraps, QKV and gate/up ranges hold whole tiles between two cut
+    ones, the tiles of O and down are cut into tens of parts and ranges end one tile and begin the next."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    qkv, o, gate_up, down = ((tiles * nkb / sms, nkb) for tiles, nkb in tc_units(MANY_UNITS))
+    for per_cta, nkb in (qkv, gate_up):
+        assert per_cta > 5 and (per_cta - 2 * (nkb - 1)) > 1          # at least one whole tile in the shortest range
+    for per_cta, nkb in (o, down):
+        assert per_cta > 2 and nkb / per_cta > 40
+    test_forms_agree_on_one_pass(MANY_UNITS, rows)
 
 
 @pytest.mark.parametrize("cfg", [RAGGED, HD128], ids=lambda c: c.name)
@@ -62,8 +86,8 @@ def test_rounds_against_oracle(batch, g_max):
 @pytest.mark.parametrize("prompt_len", [40, 47, 63, 65, 129, 200, 257, 1030, 2047, 2060, 2075])
 @pytest.mark.parametrize("cfg", [RAGGED, HD128], ids=lambda c: c.name)
 def test_prompt_kernels_against_decode_kernels(cfg, prompt_len):
-    """Prompts around the shortest the prefill kernels take, ragged last row tiles, K in parts (few tiles), two chunks of
-    positions and a window that straddles them: cache and hidden states against the decode kernels.  Those round queries
+    """Prompts from the shortest the prefill kernels take on, ragged last row tiles, two chunks of positions (and, with head
+    dimension 64, a window that straddles them): cache and hidden states against the decode kernels.  Those round queries
     and probabilities to bf16 (2^-9 each), the prefill kernels do not: 2^-7 of a vector's norm."""
     import paper_2504_05598_b200 as dl
     cfg = synth.small_variant(cfg, prompt_len=prompt_len, gen_len=4)
@@ -80,6 +104,39 @@ def test_prompt_kernels_against_decode_kernels(cfg, prompt_len):
     for a, b in zip(*got):
         assert np.linalg.norm(a - b) <= 2.0 ** -7 * np.linalg.norm(b)
     ctx.close()
+
+
+DEEP_IN = dict(d_model=4128, n_heads=4, n_kv_heads=2, head_dim=64, d_ffn=272)
+DEEP_IN128 = dict(d_model=4128, n_heads=2, n_kv_heads=1, head_dim=128, d_ffn=272)
+DEEP_OUT = dict(d_model=288, n_heads=64, n_kv_heads=4, head_dim=64, d_ffn=8208)
+WIDE = dict(d_model=2208, n_heads=18, n_kv_heads=9, head_dim=128, d_ffn=4624)
+WIDE64 = dict(d_model=2208, n_heads=36, n_kv_heads=9, head_dim=64, d_ffn=4624)
+
+
+@pytest.mark.parametrize("dims,prompt_len,splits", [
+    (DEEP_IN, 45, [(128, 4), (128, 1), (128, 4), (128, 1)]),
+    (DEEP_IN128, 200, [(128, 4), (128, 1), (128, 4), (128, 1)]),
+    (DEEP_IN, 1030, [(128, 4), (128, 1), (128, 3), (128, 1)]),
+    (DEEP_IN128, 1290, [(128, 3), (128, 1), (128, 2), (128, 1)]),
+    (DEEP_IN, 2047, [(128, 2), (128, 1), (128, 1), (128, 1)]),
+    (DEEP_OUT, 100, [(128, 1), (128, 4), (128, 1), (128, 4)]),
+    (DEEP_OUT, 2043, [(128, 1), (128, 3), (256, 1), (128, 3)]),
+    (WIDE, 300, [(128, 1), (128, 1), (256, 1), (128, 2)]),
+    (WIDE, 521, [(256, 1), (128, 1), (128, 1), (128, 1)]),
+    (WIDE, 1030, [(128, 1), (256, 1), (256, 1), (256, 1)]),
+    (WIDE64, 1107, [(256, 1), (256, 1), (256, 1), (256, 1)]),
+], ids=lambda v: str(v) if isinstance(v, int) else "")
+def test_prompt_tile_widths_and_parts_of_k(dims, prompt_len, splits):
+    """Every tile width and number of K parts that the launches choose (QKV, O, gate/up, down), at ragged rows, widths and K,
+    in one chunk: as above."""
+    import torch
+    import paper_2504_05598_b200 as dl
+    cfg = synth.small_variant(TINY, name="splits", n_layers=2, e_max=1, prompt_len=prompt_len, gen_len=4, emb_scale=10.0, gain_spread=0.1,
+                              seed=34, **dims)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    _, chunk, got = dl.debug_routes(dl.make_shape(cfg), sms, prompt_len, prompt_len)
+    assert chunk >= prompt_len and got == splits
+    test_prompt_kernels_against_decode_kernels(cfg, prompt_len)
 
 
 FIRST_PASS = """
