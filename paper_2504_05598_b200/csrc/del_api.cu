@@ -15,6 +15,7 @@ namespace {
 
 constexpr int PLAN_RING = 192;
 constexpr int CTR_RING = 4096;
+constexpr int WINDOW_MAX = 32;         // largest init_window
 constexpr int FLAG_PDL = 1, FLAG_GRAPH = 2, FLAG_TC = 4, FLAG_TIMING = 8, FLAG_ONECTA = 16, FLAG_NO_BULK_PREFILL = 32,
               FLAG_DECODE_ATTN_PREFILL = 64, FLAG_TRIM_ROWS = 128, FLAG_MMA_SYNC_PREFILL_ATTN = 256, FLAG_NO_WEIGHT_PREFETCH = 512, FLAG_TC_ROWS_ALL = 1024, FLAG_NO_TC_ROWS = 2048;
 enum { CLS_QKV = 0, CLS_ATTN, CLS_OPROJ, CLS_GATEUP, CLS_DOWN, CLS_LMHEAD, CLS_LMSTACK, CLS_OTHER, CLS_N };
@@ -229,7 +230,7 @@ int validate(const del_shape *s) {
     if (s->e_min < 1 || s->e_min > s->e_max || s->e_max >= s->n_layers) return DEL_EINVAL;
     if (s->g_min < 0 || s->g_min > s->g_max || s->g_max > DEL_MAX_GAMMA) return DEL_EINVAL;
     if (s->max_batch * (s->g_max + 1) > DEL_ROWS_MAX) return DEL_EINVAL;
-    if (s->init_window < 1 || s->init_window > 32) return DEL_EINVAL;
+    if (s->init_window < 1 || s->init_window > WINDOW_MAX) return DEL_EINVAL;
     if (!(s->omega >= 0.0 && s->omega <= 1.0)) return DEL_EINVAL;
     if (s->n_pages < 1) return DEL_EINVAL;
     return DEL_OK;
@@ -1247,10 +1248,11 @@ int del_prefill(del_ctx *c, int sq, const int32_t *prompt, int n_prompt, int max
     // chunks of <= S positions; the last chunk is exactly the window so that its hidden states stay
     // in slots 0..W-1 of the stack
     std::vector<std::pair<int, int>> chunks;
-    // From 40 positions on a prompt goes through the tensor-core prefill as a whole; shorter ones take a pass or two of the
-    // decode kernels.  us per layer, decode kernels / prefill kernels: 7B shape 36 positions 225 / 222, 45: 247 / 223, 77: 286 /
-    // 229; 1B 36: 158 / 168, 40: 168 / 169, 45: 184 / 167, 77: 239 / 181; 13B 33: 307 / 255; tiny 40: 60 / 66, 48: 68 / 67.
-    if (c->pf_ok && !(c->flags & FLAG_NO_BULK_PREFILL) && n_prompt >= 40 && n_prompt - W >= 8) {
+    // Prompts longer than the longest window go through the tensor-core prefill as a whole: the decode kernels would take two
+    // passes (the window is one of its own) where a window alone takes one, which is faster.  us per layer, decode kernels /
+    // prefill kernels: 13B shape 33 positions 304 / 234, 77: 369 / 244; 7B 33: 221 / 204, 48: 248 / 205, 77: 289 / 210;
+    // 1B 33: 142 / 130, 48: 172 / 131; 88 MB per layer 33: 136 / 113; 24 MB 33: 80 / 73; tiny 33: 59 / 48, 77: 93 / 54.
+    if (c->pf_ok && !(c->flags & FLAG_NO_BULK_PREFILL) && n_prompt > WINDOW_MAX) {
         rc = prefill_bulk(c, sq, n_prompt, n_prompt - W);
         if (rc) return rc;
     } else {

@@ -561,7 +561,7 @@ void prefill_tc_split(int epi, const Dims &D, int M, int n_sms, int *bn, int *pa
 // Positions per chunk of a prompt of n: the whole number of 128-row tiles, at most max_rows, with the smallest estimated
 // time of the four GEMMs over all chunks (a wave of tiles that is nearly empty costs as much as a full one: the 13B shape's
 // down projection has 160 tiles of 256 at 1024 rows, 240 at 1536, on 148 SMs; its 3072-position prompt
-// takes 3418 us per layer in chunks of 1024 and 2742 in chunks of 1536)
+// takes 3494 us per layer in chunks of 1024 and 3079 in chunks of 1536)
 int prefill_tc_chunk(const Dims &D, int n, int n_sms, int max_rows) {
     int best = 0;
     double best_us = 0.0;

@@ -21,8 +21,9 @@
 // and half of the columns, accumulators double-buffered.  Rotary and gate / up partners sit in other lanes; they
 // change places through shared memory.  One thread's issue latency paces each of the first three roles: with K blocks
 // of 64, two rings and ring positions by division the same loop took 0.85 us per 16 KB of weights instead of 0.33.
-// What bounds it now, 16 rows of the 7B shape: gate/up streams its 180 MB in 24 us of 30, the rest is the launch's first
-// round trip, and 2-5 us of ticket and merge at the end; the layer takes 100 us (streaming form: 140; 32 rows: 121, 251).
+// What bounds it now: HBM between a launch's first round trip and the ticket and merge at its end.  16 rows of the 7B shape,
+// launches one at a time: QKV 26, O 14, gate/up 35 (180 MB, 5.2 TB/s), down 23 us; the layer, chained and with attention,
+// takes 102 us (streaming form: 141; 32 rows: 124, 258).
 #include <cuda.h>
 
 #include <cstring>

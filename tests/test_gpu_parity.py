@@ -95,9 +95,9 @@ def test_tensor_core_prefill_against_oracle(cfg):
     o.close()
 
 
-@pytest.mark.parametrize("prompt_len", [1, 2, 39, 40, 41, 95, 96, 97])
+@pytest.mark.parametrize("prompt_len", [1, 2, 32, 33, 34, 40, 95, 96, 97])
 def test_prompt_length_edges(prompt_len):
-    """One-token prompt (window of one position), the lengths around the switch to the tensor-core prefill (40 positions),
+    """One-token prompt (window of one position), the lengths around the switch to the tensor-core prefill (33 positions),
     and around three windows of 32."""
     import oracle
     cfg = synth.small_variant(TINY, name=f"tiny_p{prompt_len}", prompt_len=prompt_len, gen_len=12, emb_scale=10.0,

@@ -83,7 +83,7 @@ def test_rounds_against_oracle(batch, g_max):
     ctx.close()
 
 
-@pytest.mark.parametrize("prompt_len", [40, 47, 63, 65, 129, 200, 257, 1030, 2047, 2060, 2075])
+@pytest.mark.parametrize("prompt_len", [33, 40, 47, 63, 65, 129, 200, 257, 1030, 2047, 2060, 2075])
 @pytest.mark.parametrize("cfg", [RAGGED, HD128], ids=lambda c: c.name)
 def test_prompt_kernels_against_decode_kernels(cfg, prompt_len):
     """Prompts from the shortest the prefill kernels take on, ragged last row tiles, two chunks of positions (and, with head
