@@ -84,12 +84,6 @@ struct del_ctx {
     WtBuffers wt = {};
     bool wt_ok = false;
     int wt_rows_min = DEL_ROWS_MAX + 1;                   // rows from which on a pass takes that form
-    // whole passes in one kernel (pass_tc.cuh): input maps for 8, 16, 32, 48, 64 rows, the layers' weights, the counters' values
-    PassTcMaps pass_maps[5];
-    PassLayer *pass_layers = nullptr;
-    int32_t *pass_count = nullptr;
-    int32_t pass_base[5] = {0};
-    bool pass_ok = false;
     bool pf_ok = false;
     int pf_rows = 0;                                      // positions the chunk buffers hold
     // mailbox of the draft loop's confidence check: pinned host memory that the finalise kernel writes directly
@@ -122,7 +116,7 @@ namespace {
 int prefill_rows(const del_shape &s) { return std::min(PF_ROWS, (s.max_seq + 127) / 128 * 128); }
 
 size_t carve_all(const del_shape &s, int pf_rows, void *base, Dims &D, Buffers &B, int &R_max, int &n_vtiles,
-                 del_round_out **out_dev, float **dbg_dev, PfArgs *pf, WtBuffers *wt, PassLayer **layers = nullptr, int32_t **count = nullptr) {
+                 del_round_out **out_dev, float **dbg_dev, PfArgs *pf, WtBuffers *wt) {
     D.L = s.n_layers; D.d = s.d_model; D.nh = s.n_heads; D.nkv = s.n_kv_heads; D.hd = s.head_dim; D.F = s.d_ffn; D.V = s.vocab;
     D.B = s.max_batch;
     // slots of the hidden stack per sequence: what a round needs (g_max + 1 rows, the prefill window), raised to
@@ -204,12 +198,8 @@ size_t carve_all(const del_shape &s, int pf_rows, void *base, Dims &D, Buffers &
     wtb.n_tickets = std::max({DEL_WT_CTAS, rowgemm_tc_tiles(EPI_QKV, D), rowgemm_tc_tiles(EPI_GATEUP, D), rowgemm_tc_tiles(EPI_DOWN, D)});
     wtb.xd = c.take<bf16>(base, (size_t)DEL_ROWS_MAX * D.d);
     wtb.xdl = c.take<bf16>(base, (size_t)DEL_ROWS_MAX * D.d);
-    wtb.part = c.take<float>(base, (size_t)rowgemm_tc_ctas(D) * 4 * DEL_ROWS_MAX * 128);
-    wtb.ticket = c.take<int32_t>(base, (size_t)wtb.n_tickets * 4);
-    PassLayer *pl = c.take<PassLayer>(base, (size_t)D.L);
-    int32_t *pc = c.take<int32_t>(base, 5);
-    if (layers) *layers = pl;
-    if (count) *count = pc;
+    wtb.part = c.take<float>(base, (size_t)rowgemm_tc_ctas(D) * 2 * DEL_ROWS_MAX * 128);
+    wtb.ticket = c.take<int32_t>(base, (size_t)wtb.n_tickets);
     if (wt) *wt = wtb;
     return (c.off + 255) & ~(size_t)255;
 }
@@ -549,81 +539,6 @@ int run_layer(del_ctx *c, const PassInfo &pi, int l, bool write_exit, bool first
     return DEL_OK;
 }
 
-// tensor maps and layer table of the passes in one kernel; false: the device cannot run them
-bool init_pass(del_ctx *c) {
-    const Dims &D = c->D;
-    int dev = 0, coop = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return false;
-    const uint64_t qd = (uint64_t)D.nh * D.hd;
-    for (int i = 0; i < 5; ++i) {
-        static const int rows[5] = {8, 16, 32, 48, 64};
-        const bf16 *x[4] = {c->wt.xd, c->B.ATT, c->B.XM, c->B.ACT}, *xl[4] = {c->wt.xdl, c->B.ATTL, c->B.XML, c->B.ACTL};
-        const uint64_t cols[4] = {(uint64_t)D.d, qd, (uint64_t)D.d, (uint64_t)D.F};
-        for (int p = 0; p < 4; ++p)
-            if (lmhead_tc_make_map(c->pass_maps[i].x[p], x[p], DEL_ROWS_MAX, cols[p], rows[i]) != 0 ||
-                lmhead_tc_make_map(c->pass_maps[i].xl[p], xl[p], DEL_ROWS_MAX, cols[p], rows[i]) != 0)
-                return false;
-    }
-    std::vector<PassLayer> t(D.L);
-    for (int l = 0; l < D.L; ++l) {
-        const del_ctx::TMap *m[7] = {&c->wt_q[l], &c->wt_k[l], &c->wt_v[l], &c->wt_o[l], &c->wt_g[l], &c->wt_u[l], &c->wt_d[l]};
-        memset(&t[l], 0, sizeof(t[l]));
-        for (int i = 0; i < 7; ++i) memcpy(t[l].w[i], m[i]->b, 128);
-        t[l].ffn_gain = c->ffn_norm[l];
-        t[l].next_gain = l + 1 < D.L ? c->attn_norm[l + 1] : nullptr;
-    }
-    return cudaMemcpyAsync(c->pass_layers, t.data(), sizeof(PassLayer) * D.L, cudaMemcpyHostToDevice, c->st) == cudaSuccess &&
-           cudaStreamSynchronize(c->st) == cudaSuccess;
-}
-
-// layers l0 .. l1 over the rows of a pass, in one kernel
-int run_pass(del_ctx *c, const PassInfo &pi, int l0, int l1, bool write_exit) {
-    const Dims &D = c->D;
-    PassTcArgs a;
-    memset(&a, 0, sizeof(a));
-    a.D = D;
-    a.B = c->B;
-    a.plan = c->plan_host[pi.plan_idx];
-    a.layers = c->pass_layers;
-    a.exit_gain = write_exit ? c->final_norm : nullptr;
-    a.xd = c->wt.xd; a.xdl = c->wt.xdl;
-    a.part = c->wt.part;
-    a.ticket = c->wt.ticket; a.n_tickets = c->wt.n_tickets;
-    a.count = c->pass_count;
-    a.l_begin = l0; a.l_end = l1;
-    const int R = pi.max_rows * (D.nh / D.nkv), n_mt = (R + 15) / 16;
-    a.n_splits = attention_splits((pi.max_kv + 15) / 16, pi.n_seg * D.nkv, n_mt >= 3 ? 4 : n_mt, c->n_sms);
-    if (c->in_round)
-        for (int i = 0; i < pi.n_seg; ++i) a.early_pos[i] = c->seq[a.plan.seg[i].seq].T;
-    for (int p = EPI_QKV; p <= EPI_DOWN; ++p) {
-        const int K = p == EPI_OPROJ ? D.nh * D.hd : (p == EPI_DOWN ? D.F : D.d);
-        a.tiles[p] = rowgemm_tc_tiles(p, D);
-        a.nkb[p] = (K + 127) / 128;
-        a.step[p] = a.tiles[p];
-    }
-    a.step[PASS_ATT] = pi.n_seg * D.nkv;
-    memcpy(a.base, c->pass_base, sizeof(a.base));
-    const int grid = std::min(c->n_sms, rowgemm_tc_ctas(D)), np = pass_tc_rows(pi.m);
-    const PassTcMaps &maps = c->pass_maps[np == 8 ? 0 : (np == 16 ? 1 : np / 16)];
-    TAG(CLS_GATEUP, 2.0 * (l1 - l0 + 1) * ((double)D.d * (D.nh + 2 * D.nkv) * D.hd + (double)D.nh * D.hd * D.d + 3.0 * D.d * D.F));
-    LAUNCH(D.hd == 64 ? launch_pass_tc_hd64(maps, a, np, grid, c->st, pdl(c)) : launch_pass_tc_hd128(maps, a, np, grid, c->st, pdl(c)));
-    // (32-bit wrap: the kernel compares differences)
-    for (int p = 0; p < 5; ++p) c->pass_base[p] = (int32_t)((uint32_t)c->pass_base[p] + (uint32_t)(l1 - l0 + 1 + (p == EPI_DOWN)) * (uint32_t)a.step[p]);
-    return DEL_OK;
-}
-
-bool use_pass(const del_ctx *c) { return c->pass_ok && !(c->flags & FLAG_NO_TC_ROWS) && (c->flags & FLAG_TC_ROWS_ALL); }
-
-int run_layers(del_ctx *c, const PassInfo &pi, int l0, int l1, bool write_exit) {
-    if (l0 > l1) return DEL_OK;
-    if (use_pass(c)) return run_pass(c, pi, l0, l1, write_exit);
-    for (int l = l0; l <= l1; ++l) {
-        const int rc = run_layer(c, pi, l, write_exit && l == l1, l == l0);
-        if (rc) return rc;
-    }
-    return DEL_OK;
-}
-
 // sequences of a call with their round parameters
 struct Job { int seq, E, g; int stopped = 0; };
 
@@ -691,9 +606,10 @@ int launch_draft_step(del_ctx *c, const DraftStep &st, const std::vector<int> &E
     for (size_t e = 0; e < Es.size(); ++e) {
         if (st.sub_idx[e] < 0) break;
         const PassInfo pi = pass_info(c, st.sub_idx[e]);
-        const int rc = run_layers(c, pi, l, Es[e], true);
-        if (rc) return rc;
-        l = Es[e] + 1;
+        for (const int l0 = l; l <= Es[e]; ++l) {
+            int rc = run_layer(c, pi, l, l == Es[e], l == l0);
+            if (rc) return rc;
+        }
     }
     GemmArgs a = gemm_base(c, full.plan_idx, 0);
     a.K = c->D.d;
@@ -938,9 +854,10 @@ int enqueue_verify(del_ctx *c, const std::vector<Job> &jobs) {
         const int l_last = k < Es.size() ? Es[k] : c->D.L;
         if (idx[k] < 0) { l = l_last + 1; continue; }
         const PassInfo pi = pass_info(c, idx[k]);
-        rc = run_layers(c, pi, l, l_last, false);
-        if (rc) return rc;
-        l = l_last + 1;
+        for (const int l0 = l; l <= l_last; ++l) {
+            rc = run_layer(c, pi, l, false, l == l0);
+            if (rc) return rc;
+        }
     }
     return DEL_OK;
 }
@@ -1103,11 +1020,7 @@ int read_out(del_ctx *c) {
         // a bounded device-side wait expired; clear the word so that the context stays usable
         snprintf(c->err, sizeof(c->err), "device wait expired (code %d)", *err_host);
         cudaMemsetAsync(c->B.ERR, 0, sizeof(int32_t), c->st);
-        // a launch that gave up leaves arrivals behind
-        cudaMemsetAsync(c->wt.ticket, 0, sizeof(int32_t) * c->wt.n_tickets * 4, c->st);
-        cudaMemsetAsync(c->B.ACNT, 0, sizeof(int32_t) * DEL_SEQ_MAX * c->D.nkv, c->st);
-        cudaMemsetAsync(c->pass_count, 0, sizeof(int32_t) * 5, c->st);
-        memset(c->pass_base, 0, sizeof(c->pass_base));
+        cudaMemsetAsync(c->wt.ticket, 0, sizeof(int32_t) * c->wt.n_tickets, c->st);      // a launch that gave up leaves arrivals behind
         return DEL_ETIMEOUT;
     }
     return DEL_OK;
@@ -1180,7 +1093,7 @@ int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const 
     if (!c) return DEL_ENOSPC;
     c->sh = *shape;
     c->pf_rows = pf_rows;
-    carve_all(*shape, pf_rows, workspace, c->D, c->B, c->R_max, c->n_vtiles, &c->out_dev, &c->dbg_dev, &c->pf, &c->wt, &c->pass_layers, &c->pass_count);
+    carve_all(*shape, pf_rows, workspace, c->D, c->B, c->R_max, c->n_vtiles, &c->out_dev, &c->dbg_dev, &c->pf, &c->wt);
     c->B.KP = (bf16 *)kv->k_pages; c->B.VP = (bf16 *)kv->v_pages; c->B.PT = kv->page_table;
     c->B.rope_cos = w->rope_cos; c->B.rope_sin = w->rope_sin;
     c->tok_emb = (const bf16 *)w->tok_emb; c->final_norm = (const bf16 *)w->final_norm; c->lm_head = (const bf16 *)w->lm_head;
@@ -1281,11 +1194,6 @@ int del_init(del_ctx **out, const del_shape *shape, const del_weights *w, const 
             del_destroy(c);
             return DEL_ECUDA;
         }
-        c->pass_ok = c->wt_ok && init_pass(c);
-        if (c->pass_ok && (c->D.hd == 64 ? pass_tc_prepare_hd64() : pass_tc_prepare_hd128()) != cudaSuccess) {
-            del_destroy(c);
-            return DEL_ECUDA;
-        }
         c->pfa_ok = ok && prefill_attention_tc_supported(c->D) &&
                     lmhead_tc_make_map(c->pf_q.b, c->pf.Q, pf_rows, qd, 128) == 0 &&
                     lmhead_tc_make_map(c->pf_ql.b, c->pf.QL, pf_rows, qd, 128) == 0 &&
@@ -1344,10 +1252,7 @@ int del_prefill(del_ctx *c, int sq, const int32_t *prompt, int n_prompt, int max
     // passes (the window is one of its own) where a window alone takes one, which is faster.  us per layer, decode kernels /
     // prefill kernels: 13B shape 33 positions 304 / 234, 77: 369 / 244; 7B 33: 221 / 204, 48: 248 / 205, 77: 289 / 210;
     // 1B 33: 142 / 130, 48: 172 / 131; 88 MB per layer 33: 136 / 113; 24 MB 33: 80 / 73; tiny 33: 59 / 48, 77: 93 / 54.
-    const bool one_pass = n_prompt > W && n_prompt <= DEL_ROWS_MAX && use_pass(c) && !(c->flags & FLAG_NO_BULK_PREFILL);
-    if (one_pass) {
-        chunks.push_back({0, n_prompt});
-    } else if (c->pf_ok && !(c->flags & FLAG_NO_BULK_PREFILL) && n_prompt > WINDOW_MAX) {
+    if (c->pf_ok && !(c->flags & FLAG_NO_BULK_PREFILL) && n_prompt > WINDOW_MAX) {
         rc = prefill_bulk(c, sq, n_prompt, n_prompt - W);
         if (rc) return rc;
     } else {
@@ -1361,18 +1266,17 @@ int del_prefill(del_ctx *c, int sq, const int32_t *prompt, int n_prompt, int max
         PlanBatch pb(c);
         int idx;
         s.T = ch.first;                      // rows are addressed relative to the committed length
-        PassPlan *plan = pb.add(&idx);
-        fill_plan(c, plan, {RowSpec{sq, 0, ch.second}}, true);
-        if (one_pass)               // the window in slots 0..W-1, the positions before it in the slots behind
-            for (int i = 0; i < n_prompt; ++i) plan->rows[i].slot = i >= n_prompt - W ? i - (n_prompt - W) : W + i;
+        fill_plan(c, pb.add(&idx), {RowSpec{sq, 0, ch.second}}, true);
         rc = plan_commit(c, pb);
         if (rc) return rc;
         CtlArgs ca = ctl_base(c, idx);
         ca.tok_src = c->B.PROMPT_ALL;
         LAUNCH(launch_embed(ca, ch.second, c->st, pdl(c)));
         const PassInfo pi = pass_info(c, idx);
-        rc = run_layers(c, pi, 1, c->D.L, false);
-        if (rc) return rc;
+        for (int l = 1; l <= c->D.L; ++l) {
+            rc = run_layer(c, pi, l, false, l == 1);
+            if (rc) return rc;
+        }
     }
     s.T = n_prompt;
     s.active = true;

@@ -63,40 +63,6 @@ cudaError_t rowgemm_tc_prepare();
 cudaError_t launch_rowgemm_tc(int epi, const GemmArgs &a, const void *map_w0, const void *map_w1, const void *map_w2, const void *map_x,
                               const void *map_xl, bool dense, const WtBuffers &b, int n_sms, cudaStream_t st, bool pdl);
 
-// A pass through several layers in one kernel (pass_tc.cuh)
-#define PASS_ATT 4             // index of attention's counter behind the four GEMM phases (EPI_QKV .. EPI_DOWN)
-struct alignas(64) PassLayer { // one layer's weights; an array of them lies in the workspace
-    unsigned char w[7][128];   // tensor maps: Wq, Wk, Wv, Wo, gate, up, down (boxes of 128 rows, gate and up 64)
-    const bf16 *ffn_gain, *next_gain;      // ffn norm; the next layer's attention norm (nullptr: last layer)
-    unsigned char pad[112];
-};
-struct PassTcMaps {            // inputs of the four phases by row of the pass, high and low parts; boxes of as many rows as the kernel takes
-    alignas(64) unsigned char x[4][128];
-    alignas(64) unsigned char xl[4][128];
-};
-struct PassTcArgs {
-    Dims D;
-    Buffers B;
-    PassPlan plan;
-    const PassLayer *layers;
-    const bf16 *exit_gain;     // final norm: layer l_end also leaves the exit head's input (nullptr: it does not)
-    bf16 *xd, *xdl;            // [ROWS][d] a layer's input by row of the pass
-    float *part;               // [2][CTAs][2][NP / 8][128][8] partial sums of the cut tiles, alternating from phase to phase
-    int32_t *ticket;           // [4][n_tickets] arrivals at a cut tile; zero between launches
-    int32_t *count;            // [5] finished tiles of the phases so far
-    int32_t n_tickets;
-    int32_t l_begin, l_end;    // 1-based layers of the launch
-    int32_t n_splits;          // key-range splits of attention
-    int32_t tiles[4], nkb[4];  // tiles and K blocks of the phases
-    int32_t base[5], step[5];  // the counters' values before the launch, and what a layer adds
-    int32_t early_pos[DEL_SEQ_MAX];        // as in AttnArgs
-};
-inline int pass_tc_rows(int m) { return m <= 8 ? 8 : (m <= 16 ? 16 : (m <= 32 ? 32 : (m <= 48 ? 48 : 64))); }
-cudaError_t pass_tc_prepare_hd64();        // loads the kernels onto the current device (rowgemm_tc_prepare)
-cudaError_t pass_tc_prepare_hd128();
-cudaError_t launch_pass_tc_hd64(const PassTcMaps &maps, const PassTcArgs &w, int np, int grid, cudaStream_t st, bool pdl);
-cudaError_t launch_pass_tc_hd128(const PassTcMaps &maps, const PassTcArgs &w, int np, int grid, cudaStream_t st, bool pdl);
-
 struct AttnArgs {
     Dims D;
     Buffers B;
