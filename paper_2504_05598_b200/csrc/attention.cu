@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(NW * 32) attention_kernel(const __grid_constan
     // several query tiles share the pages through shared memory; a single tile loads its fragments directly
     const int n_mt = (seg.nrows * (a.D.nh / a.D.nkv) + 15) >> 4;
     if (n_mt >= 2) attn::partial_staged<HD>(v, reinterpret_cast<unsigned char *>(sm), seg, kvh, p_begin, p_end, 0, 0x7fffffff, split, n_splits);
-    else attn::partial<HD>(attn::WholeCta(), v, sm, seg, kvh, p_begin, p_end, 0, 0x7fffffff, split, n_splits);
+    else attn::partial<HD>(v, sm, seg, kvh, p_begin, p_end, 0, 0x7fffffff, split, n_splits);
 
     if (n_splits > 1) {
         // The CTA's partial states are published by one release-acquire ticket: the barrier orders every thread's
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(NW * 32) attention_kernel(const __grid_constan
             if (s_last) a.B.ACNT[blockIdx.z * a.D.nkv + kvh] = 0;     // ready for the next launch
         }
         __syncthreads();
-        if (s_last) attn::merge_slots<HD, attn::WholeCta>(v, seg, kvh, n_splits);
+        if (s_last) attn::merge_slots<HD>(v, seg, kvh, n_splits);
     }
 }
 

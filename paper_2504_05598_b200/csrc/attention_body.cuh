@@ -1,8 +1,6 @@
-// Device-side building blocks of the paged multi-query attention: of its own kernel (attention.cu) and of the kernel that
-// runs whole layers (pass_tc.cuh).  Both give 8 warps to a task; a policy says which threads they are, how they meet and how
-// they wait for the queries (WholeCta below; EpiWarps there).
+// Device-side building blocks of the paged multi-query attention kernel (attention.cu).
 //
-// partial / partial_staged contain the wait for the producer (WholeCta: programmatic dependent launch): what they
+// partial / partial_staged contain the kernel's wait for its producer (programmatic dependent launch): what they
 // read before it does not depend on the producer.
 //   attn::partial         one CTA walks a range of key pages for one (segment, kv head) and leaves, per
 //                         query row and head, an online-softmax state (max, sum, unnormalised output):
@@ -46,14 +44,6 @@ __device__ __forceinline__ void split_row(int rr, int ms, int &hq, int &i) {
 
 constexpr float LOG2E = 1.4426950408889634f;
 
-// 8 warps = the whole CTA of the attention kernel
-struct WholeCta {
-    static constexpr int T0 = 0;              // first thread
-    static constexpr int FEW = 1, MANY = 1;   // parts (of the head dimension) in which the warps' outputs are merged: up to 8 rows, more
-    __device__ __forceinline__ void sync() const { __syncthreads(); }
-    __device__ __forceinline__ bool ready(const AttnView &a) const;
-};
-
 // Every CTA of the launch requests its share of the regions in pieces of 32 KB, one piece per lane of its last warp
 // (called once the warps' own early cache reads have been issued, before the wait for the producer kernel).
 __device__ __forceinline__ void prefetch_weights(const AttnPrefetch &pf) {
@@ -70,22 +60,13 @@ __device__ __forceinline__ void prefetch_weights(const AttnPrefetch &pf) {
         }
     }
 }
-__device__ __forceinline__ bool WholeCta::ready(const AttnView &a) const {
-    prefetch_weights(*a.pf);
-    pdl_wait();
-    return true;
-}
-constexpr int NW = 8;                 // warps per task
+constexpr int NW = 8;                 // warps per CTA
 constexpr int PG = 4;                 // page ids fetched ahead per warp
 constexpr int MAX_SLOTS = 16;
 
-// shared memory of tile_end: up to 8 rows [8 warps][8][hd / FEW] and (max, sum); more [hd / 8 / MANY][8 warps][32] float4 and 8 * 32 float4
-template <typename Pol> __host__ __device__ constexpr size_t merge_bytes(int hd) {
-    const size_t few = sizeof(float) * ((size_t)NW * 8 * (hd / Pol::FEW) + NW * 8 * 2);
-    const size_t many = sizeof(float) * ((size_t)NW * 32 * (hd / 8 / Pol::MANY) * 4 + (size_t)NW * 32 * 4);
-    return few > many ? few : many;
+__host__ __device__ constexpr size_t smem_bytes(int hd) {
+    return sizeof(float) * ((size_t)NW * 32 * (hd / 8) * 4 + (size_t)NW * 32 * 4);
 }
-__host__ __device__ constexpr size_t smem_bytes(int hd) { return merge_bytes<WholeCta>(hd); }
 
 // Per-thread view of one 16-row query tile: which rows of the segment the thread's two MMA rows are,
 // their query fragments, and the running softmax state.
@@ -169,13 +150,14 @@ __device__ __forceinline__ void page_update(TileState<HD> &ts, const uint4 (&kf)
 
 // The warps of each query tile merge their states through shared memory (every warp of the CTA merges
 // some output column tiles) and write the result: normalised to ATT when n_slots == 1, otherwise as a
-// partial state to slot `slot`.  it = iteration over groups of P concurrent query tiles.  The outputs pass in
-// Pol::FEW or Pol::MANY parts, which bounds the memory: see merge_bytes.
-template <int HD, typename Pol>
-__device__ __forceinline__ void tile_end(const Pol &pol, TileState<HD> &ts, const AttnView &a, float *sm, const Segment seg, int kvh, int it,
+// partial state to slot `slot`.  it = iteration over groups of P concurrent query tiles.
+template <int HD>
+__device__ __forceinline__ void tile_end(TileState<HD> &ts, const AttnView &a, float *sm, const Segment seg, int kvh, int it,
                                          int P, int n_mt, int slot, int n_slots) {
     constexpr int NJ = HD / 8;
-    const int tid = threadIdx.x - Pol::T0, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    float *sm_o = sm;                               // [NJ][NW][32] float4
+    float *sm_ml = sm + NW * 32 * NJ * 4;           // [NW][32] float4
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int ms = seg.nrows, group = a.D.nh / a.D.nkv, R = ms * group, qdim = a.D.nh * HD;
     const int n_kl = NW / P;
 #pragma unroll
@@ -185,120 +167,110 @@ __device__ __forceinline__ void tile_end(const Pol &pol, TileState<HD> &ts, cons
     }
     if (R <= 8) {
         // Few query rows (one sequence drafting or verifying a handful of tokens): only rows 0..R-1 of the tile
-        // carry data, i.e. MMA rows g < R and none of the rows g + 8.  Merge just those: [warp][row][HC] floats.
-        constexpr int HC = HD / Pol::FEW, JC = HC / 8;
-        float *so = sm;                             // [NW][R][HC]
-        float *sml = sm + NW * 8 * HC;              // [NW][8] (max, sum)
-        if (g < R && t == 0) *reinterpret_cast<float2 *>(sml + (warp * 8 + g) * 2) = make_float2(ts.m_run[0], ts.l_run[0]);
+        // carry data, i.e. MMA rows g < R and none of the rows g + 8.  Merge just those: [warp][row][HD] floats.
+        float *so = sm;                             // [NW][R][HD]
+        float *sml = sm + NW * 8 * HD;              // [NW][8] (max, sum)
+        if (g < R) {
+            float *dst = so + ((size_t)warp * R + g) * HD + 2 * t;
 #pragma unroll
-        for (int part = 0; part < Pol::FEW; ++part) {
-            if (g < R) {
-                float *dst = so + ((size_t)warp * R + g) * HC + 2 * t;
-#pragma unroll
-                for (int j = 0; j < JC; ++j) *reinterpret_cast<float2 *>(dst + 8 * j) = make_float2(ts.O[part * JC + j][0], ts.O[part * JC + j][1]);
-            }
-            pol.sync();
-            for (int e = tid; e < R * (HC / 2); e += NW * 32) {
-                const int row = e / (HC / 2), cc = (e - row * (HC / 2)) * 2, col = part * HC + cc;
-                float M = -INFINITY;
-#pragma unroll
-                for (int w2 = 0; w2 < NW; ++w2) M = fmaxf(M, sml[(w2 * 8 + row) * 2]);
-                const float b = M == -INFINITY ? 0.f : M;
-                float L = 0.f, o0 = 0.f, o1 = 0.f;
-#pragma unroll
-                for (int w2 = 0; w2 < NW; ++w2) {
-                    const float2 ml = *reinterpret_cast<const float2 *>(sml + (w2 * 8 + row) * 2);
-                    const float f = exp2f(ml.x - b);
-                    const float2 ov = *reinterpret_cast<const float2 *>(so + ((size_t)w2 * R + row) * HC + cc);
-                    L += ml.y * f;
-                    o0 += ov.x * f;
-                    o1 += ov.y * f;
-                }
-                int hq, i;
-                split_row(row, ms, hq, i);
-                const int c = seg.row0 + i, qh = kvh * group + hq;
-                if (n_slots == 1) {
-                    const float inv = 1.f / L;
-                    uint32_t hi, lo;
-                    split_bf16x2(o0 * inv, o1 * inv, hi, lo);
-                    *reinterpret_cast<uint32_t *>(a.B.ATT + (size_t)c * qdim + qh * HD + col) = hi;
-                    *reinterpret_cast<uint32_t *>(a.B.ATTL + (size_t)c * qdim + qh * HD + col) = lo;
-                } else {
-                    const size_t pi = ((size_t)c * a.D.nh + qh) * n_slots + slot;
-                    *reinterpret_cast<float2 *>(a.B.APO + pi * HD + col) = make_float2(o0, o1);
-                    if (col == 0) *reinterpret_cast<float2 *>(a.B.APML + pi * 2) = make_float2(M, L);
-                }
-            }
-            pol.sync();
+            for (int j = 0; j < NJ; ++j) *reinterpret_cast<float2 *>(dst + 8 * j) = make_float2(ts.O[j][0], ts.O[j][1]);
+            if (t == 0) *reinterpret_cast<float2 *>(sml + (warp * 8 + g) * 2) = make_float2(ts.m_run[0], ts.l_run[0]);
         }
+        __syncthreads();
+        for (int e = tid; e < R * (HD / 2); e += NW * 32) {
+            const int row = e / (HD / 2), col = (e - row * (HD / 2)) * 2;
+            float M = -INFINITY;
+#pragma unroll
+            for (int w2 = 0; w2 < NW; ++w2) M = fmaxf(M, sml[(w2 * 8 + row) * 2]);
+            const float b = M == -INFINITY ? 0.f : M;
+            float L = 0.f, o0 = 0.f, o1 = 0.f;
+#pragma unroll
+            for (int w2 = 0; w2 < NW; ++w2) {
+                const float2 ml = *reinterpret_cast<const float2 *>(sml + (w2 * 8 + row) * 2);
+                const float f = exp2f(ml.x - b);
+                const float2 ov = *reinterpret_cast<const float2 *>(so + ((size_t)w2 * R + row) * HD + col);
+                L += ml.y * f;
+                o0 += ov.x * f;
+                o1 += ov.y * f;
+            }
+            int hq, i;
+            split_row(row, ms, hq, i);
+            const int c = seg.row0 + i, qh = kvh * group + hq;
+            if (n_slots == 1) {
+                const float inv = 1.f / L;
+                uint32_t hi, lo;
+                split_bf16x2(o0 * inv, o1 * inv, hi, lo);
+                *reinterpret_cast<uint32_t *>(a.B.ATT + (size_t)c * qdim + qh * HD + col) = hi;
+                *reinterpret_cast<uint32_t *>(a.B.ATTL + (size_t)c * qdim + qh * HD + col) = lo;
+            } else {
+                const size_t pi = ((size_t)c * a.D.nh + qh) * n_slots + slot;
+                *reinterpret_cast<float2 *>(a.B.APO + pi * HD + col) = make_float2(o0, o1);
+                if (col == 0) *reinterpret_cast<float2 *>(a.B.APML + pi * 2) = make_float2(M, L);
+            }
+        }
+        __syncthreads();
         return;
     }
-    constexpr int JC = NJ / Pol::MANY;
-    float *sm_o = sm;                               // [JC][NW][32] float4
-    float *sm_ml = sm + NW * 32 * JC * 4;           // [NW][32] float4
+    // layout [column tile][warp][lane]: consecutive lanes write consecutive 16-byte words
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+        *reinterpret_cast<float4 *>(sm_o + (size_t)((j * NW + warp) * 32 + lane) * 4) =
+            make_float4(ts.O[j][0], ts.O[j][1], ts.O[j][2], ts.O[j][3]);
     *reinterpret_cast<float4 *>(sm_ml + (warp * 32 + lane) * 4) = make_float4(ts.m_run[0], ts.l_run[0], ts.m_run[1], ts.l_run[1]);
+    __syncthreads();
+    for (int task = warp; task < P * NJ; task += NW) {
+        const int mp = task / NJ, j = task - mp * NJ;      // query-tile slot of this iteration, column tile
+        const int mt2 = it * P + mp;
+        if (mt2 >= n_mt) continue;
+        float M0 = -INFINITY, M1 = -INFINITY;
+        for (int k2 = 0; k2 < n_kl; ++k2) {
+            const float4 ml = *reinterpret_cast<const float4 *>(sm_ml + ((mp + k2 * P) * 32 + lane) * 4);
+            M0 = fmaxf(M0, ml.x);
+            M1 = fmaxf(M1, ml.z);
+        }
+        const float b0 = M0 == -INFINITY ? 0.f : M0, b1 = M1 == -INFINITY ? 0.f : M1;
+        float L0 = 0.f, L1 = 0.f, o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
+        for (int k2 = 0; k2 < n_kl; ++k2) {
+            const int w2 = mp + k2 * P;
+            const float4 ml = *reinterpret_cast<const float4 *>(sm_ml + (w2 * 32 + lane) * 4);
+            const float f0 = exp2f(ml.x - b0), f1 = exp2f(ml.z - b1);
+            L0 += ml.y * f0;
+            L1 += ml.w * f1;
+            const float4 ov = *reinterpret_cast<const float4 *>(sm_o + (size_t)((j * NW + w2) * 32 + lane) * 4);
+            o0 += ov.x * f0; o1 += ov.y * f0; o2 += ov.z * f1; o3 += ov.w * f1;
+        }
+        const float Mv[2] = {M0, M1}, Lv[2] = {L0, L1}, ov2[2][2] = {{o0, o1}, {o2, o3}};
 #pragma unroll
-    for (int part = 0; part < Pol::MANY; ++part) {
-        // layout [column tile][warp][lane]: consecutive lanes write consecutive 16-byte words
-#pragma unroll
-        for (int j = 0; j < JC; ++j)
-            *reinterpret_cast<float4 *>(sm_o + (size_t)((j * NW + warp) * 32 + lane) * 4) =
-                make_float4(ts.O[part * JC + j][0], ts.O[part * JC + j][1], ts.O[part * JC + j][2], ts.O[part * JC + j][3]);
-        pol.sync();
-        for (int task = warp; task < P * JC; task += NW) {
-            const int mp = task / JC, jl = task - mp * JC, j = part * JC + jl;      // query-tile slot of this iteration, column tile
-            const int mt2 = it * P + mp;
-            if (mt2 >= n_mt) continue;
-            float M0 = -INFINITY, M1 = -INFINITY;
-            for (int k2 = 0; k2 < n_kl; ++k2) {
-                const float4 ml = *reinterpret_cast<const float4 *>(sm_ml + ((mp + k2 * P) * 32 + lane) * 4);
-                M0 = fmaxf(M0, ml.x);
-                M1 = fmaxf(M1, ml.z);
-            }
-            const float b0 = M0 == -INFINITY ? 0.f : M0, b1 = M1 == -INFINITY ? 0.f : M1;
-            float L0 = 0.f, L1 = 0.f, o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
-            for (int k2 = 0; k2 < n_kl; ++k2) {
-                const int w2 = mp + k2 * P;
-                const float4 ml = *reinterpret_cast<const float4 *>(sm_ml + (w2 * 32 + lane) * 4);
-                const float f0 = exp2f(ml.x - b0), f1 = exp2f(ml.z - b1);
-                L0 += ml.y * f0;
-                L1 += ml.w * f1;
-                const float4 ov = *reinterpret_cast<const float4 *>(sm_o + (size_t)((jl * NW + w2) * 32 + lane) * 4);
-                o0 += ov.x * f0; o1 += ov.y * f0; o2 += ov.z * f1; o3 += ov.w * f1;
-            }
-            const float Mv[2] = {M0, M1}, Lv[2] = {L0, L1}, ov2[2][2] = {{o0, o1}, {o2, o3}};
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int r2 = mt2 * 16 + g + 8 * h;
-                if (r2 >= R) continue;
-                int hq, i;
-                split_row(r2, ms, hq, i);
-                const int c = seg.row0 + i, qh = kvh * group + hq;
-                if (n_slots == 1) {
-                    const float inv = 1.f / Lv[h];
-                    uint32_t hi, lo;
-                    split_bf16x2(ov2[h][0] * inv, ov2[h][1] * inv, hi, lo);
-                    *reinterpret_cast<uint32_t *>(a.B.ATT + (size_t)c * qdim + qh * HD + 8 * j + 2 * t) = hi;
-                    *reinterpret_cast<uint32_t *>(a.B.ATTL + (size_t)c * qdim + qh * HD + 8 * j + 2 * t) = lo;
-                } else {
-                    const size_t pi = ((size_t)c * a.D.nh + qh) * n_slots + slot;
-                    *reinterpret_cast<float2 *>(a.B.APO + pi * HD + 8 * j + 2 * t) = make_float2(ov2[h][0], ov2[h][1]);
-                    if (j == 0 && t == 0) *reinterpret_cast<float2 *>(a.B.APML + pi * 2) = make_float2(Mv[h], Lv[h]);
-                }
+        for (int h = 0; h < 2; ++h) {
+            const int r2 = mt2 * 16 + g + 8 * h;
+            if (r2 >= R) continue;
+            int hq, i;
+            split_row(r2, ms, hq, i);
+            const int c = seg.row0 + i, qh = kvh * group + hq;
+            if (n_slots == 1) {
+                const float inv = 1.f / Lv[h];
+                uint32_t hi, lo;
+                split_bf16x2(ov2[h][0] * inv, ov2[h][1] * inv, hi, lo);
+                *reinterpret_cast<uint32_t *>(a.B.ATT + (size_t)c * qdim + qh * HD + 8 * j + 2 * t) = hi;
+                *reinterpret_cast<uint32_t *>(a.B.ATTL + (size_t)c * qdim + qh * HD + 8 * j + 2 * t) = lo;
+            } else {
+                const size_t pi = ((size_t)c * a.D.nh + qh) * n_slots + slot;
+                *reinterpret_cast<float2 *>(a.B.APO + pi * HD + 8 * j + 2 * t) = make_float2(ov2[h][0], ov2[h][1]);
+                if (j == 0 && t == 0) *reinterpret_cast<float2 *>(a.B.APML + pi * 2) = make_float2(Mv[h], Lv[h]);
             }
         }
-        pol.sync();
     }
+    __syncthreads();
 }
 
 // Keys of pages [p_begin, p_end) that lie in [k_lo, k_hi] and are not in the future of the query row,
-// fragments loaded straight from global memory.  `sm`: merge_bytes<Pol>(HD) of shared memory; all 256 threads call.
-// false: the wait for the queries gave up (in all threads alike).
-template <int HD, typename Pol>
-__device__ __forceinline__ bool partial(const Pol &pol, const AttnView &a, float *sm, const Segment seg, int kvh, int p_begin, int p_end,
+// fragments loaded straight from global memory.  `sm` is the CTA's dynamic shared memory
+// (smem_bytes(HD)); all 256 threads call.
+template <int HD>
+__device__ __forceinline__ void partial(const AttnView &a, float *sm, const Segment seg, int kvh, int p_begin, int p_end,
                                         int k_lo, int k_hi, int slot, int n_slots) {
     constexpr int KS = HD / 32, NJ = HD / 8;
-    const int warp = (threadIdx.x - Pol::T0) >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int R = seg.nrows * (a.D.nh / a.D.nkv), n_mt = (R + 15) >> 4;
     const int P = n_mt >= 3 ? 4 : n_mt;             // query tiles handled concurrently: 1, 2 or 4
     const int n_kl = NW / P, kl = warp / P;
@@ -335,7 +307,8 @@ __device__ __forceinline__ bool partial(const Pol &pol, const AttnView &a, float
             l2_prefetch_bulk(a.B.VP + off, 16 * HD * 2);
         }
     }
-    if (!pol.ready(a)) return false;
+    prefetch_weights(*a.pf);
+    pdl_wait();
 
     for (int it = 0; it < n_iter; ++it) {
         const int mt = it * P + warp % P;
@@ -369,9 +342,8 @@ __device__ __forceinline__ bool partial(const Pol &pol, const AttnView &a, float
                 }
             }
         }
-        tile_end<HD>(pol, ts, a, sm, seg, kvh, it, P, n_mt, slot, n_slots);
+        tile_end<HD>(ts, a, sm, seg, kvh, it, P, n_mt, slot, n_slots);
     }
-    return true;
 }
 
 // ---- staged variant: the key/value pages travel to shared memory with asynchronous copies
@@ -417,7 +389,8 @@ __device__ __forceinline__ void partial_staged(const AttnView &a, unsigned char 
     const int n_pages = max(p_end - p_begin, 0), n_chunks = (n_pages + CH - 1) / CH;
     const int n_iter = (n_mt + P - 1) / P;          // groups of P concurrent query tiles; each group stages the pages again
 
-    WholeCta().ready(a);
+    prefetch_weights(*a.pf);
+    pdl_wait();
     // every thread copies the same pieces of every page: 2*HD 16-byte pieces of keys, 2*HD of values
     auto issue = [&](int c) {
         if (c < n_chunks) {
@@ -480,7 +453,7 @@ __device__ __forceinline__ void partial_staged(const AttnView &a, unsigned char 
     }
     cp_async_wait<0>();
     __syncthreads();                                 // the merge below reuses the staging memory
-    tile_end<HD>(WholeCta(), ts, a, reinterpret_cast<float *>(smem), seg, kvh, it, P, n_mt, slot, n_slots);   // ends with a barrier
+    tile_end<HD>(ts, a, reinterpret_cast<float *>(smem), seg, kvh, it, P, n_mt, slot, n_slots);   // ends with a barrier
     }
 }
 
@@ -488,11 +461,11 @@ __device__ __forceinline__ void partial_staged(const AttnView &a, unsigned char 
 // normalised bf16 result.  The caller has made the slots visible (fence + barrier / arrival counter).
 // NS = compile-time bound on the slots, UE = elements a thread works on at once: the loads of an iteration
 // (UE * NS partial states) are all in flight together.
-template <int HD, int NS, int UE, typename Pol>
+template <int HD, int NS, int UE>
 __device__ __forceinline__ void merge_slots_n(const AttnView &a, const Segment seg, int kvh, int n_slots) {
     const int ms = seg.nrows, group = a.D.nh / a.D.nkv, R = ms * group, qdim = a.D.nh * HD;
     const int n_el = R * (HD / 4);
-    for (int e0 = threadIdx.x - Pol::T0; e0 < n_el; e0 += NW * 32 * UE) {
+    for (int e0 = threadIdx.x; e0 < n_el; e0 += NW * 32 * UE) {
         uint2 mlv[UE][NS];
         uint4 ovv[UE][NS];
         size_t out_off[UE];
@@ -544,20 +517,20 @@ __device__ __forceinline__ void merge_slots_n(const AttnView &a, const Segment s
     }
 }
 
-template <int HD, typename Pol>
+template <int HD>
 __device__ __forceinline__ void merge_slots(const AttnView &a, const Segment seg, int kvh, int n_slots) {
     // a decode-sized segment has at most one element per thread: one element per thread (least index arithmetic in
     // front of the loads) and no more loads than the split count needs (1 % of a round against always loading
     // 16 clamped slots); large segments (prefill passes) batch several elements per thread
     const int n_el = seg.nrows * (a.D.nh / a.D.nkv) * (HD / 4);
     if (n_el <= NW * 32) {
-        if (n_slots <= 2) merge_slots_n<HD, 2, 1, Pol>(a, seg, kvh, n_slots);
-        else if (n_slots <= 4) merge_slots_n<HD, 4, 1, Pol>(a, seg, kvh, n_slots);
-        else if (n_slots <= 8) merge_slots_n<HD, 8, 1, Pol>(a, seg, kvh, n_slots);
-        else merge_slots_n<HD, 16, 1, Pol>(a, seg, kvh, n_slots);
-    } else if (n_slots > 8) merge_slots_n<HD, 16, 1, Pol>(a, seg, kvh, n_slots);
-    else if (n_slots <= 4) merge_slots_n<HD, 4, 4, Pol>(a, seg, kvh, n_slots);
-    else merge_slots_n<HD, 8, 2, Pol>(a, seg, kvh, n_slots);
+        if (n_slots <= 2) merge_slots_n<HD, 2, 1>(a, seg, kvh, n_slots);
+        else if (n_slots <= 4) merge_slots_n<HD, 4, 1>(a, seg, kvh, n_slots);
+        else if (n_slots <= 8) merge_slots_n<HD, 8, 1>(a, seg, kvh, n_slots);
+        else merge_slots_n<HD, 16, 1>(a, seg, kvh, n_slots);
+    } else if (n_slots > 8) merge_slots_n<HD, 16, 1>(a, seg, kvh, n_slots);
+    else if (n_slots <= 4) merge_slots_n<HD, 4, 4>(a, seg, kvh, n_slots);
+    else merge_slots_n<HD, 8, 2>(a, seg, kvh, n_slots);
 }
 
 }  // namespace attn
