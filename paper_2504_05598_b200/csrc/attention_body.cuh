@@ -65,7 +65,7 @@ constexpr int PG = 4;                 // page ids fetched ahead per warp
 constexpr int MAX_SLOTS = 16;
 
 __host__ __device__ constexpr size_t smem_bytes(int hd) {
-    return sizeof(float) * ((size_t)NW * 32 * (hd / 8) * 4 + (size_t)NW * 32 * 4);
+    return sizeof(float) * ((size_t)NW * 16 * (hd + 8) + (size_t)NW * 16 * 2);
 }
 
 // Per-thread view of one 16-row query tile: which rows of the segment the thread's two MMA rows are,
@@ -148,15 +148,15 @@ __device__ __forceinline__ void page_update(TileState<HD> &ts, const uint4 (&kf)
     for (int j = 0; j < NJ; ++j) mma_bf16_16816(ts.O[j], pa0, pa1, pa2, pa3, vf[j].x, vf[j].y);
 }
 
-// The warps of each query tile merge their states through shared memory (every warp of the CTA merges
-// some output column tiles) and write the result: normalised to ATT when n_slots == 1, otherwise as a
-// partial state to slot `slot`.  it = iteration over groups of P concurrent query tiles.
+// The warps of each query tile merge their states through shared memory and the result is written: normalised to ATT when
+// n_slots == 1, otherwise as a partial state to slot `slot`.  it = iteration over groups of P concurrent query tiles.
+// The code for more than 8 rows has rolled loops: it runs once per launch, and fetching its instructions costs more than
+// executing them (the weight stream of a layer evicts them from L2).  Four sequences of 4 + 1 rows, 8B shape: 7.13 -> 6.93 ms
+// per round together with merge_slots.
 template <int HD>
 __device__ __forceinline__ void tile_end(TileState<HD> &ts, const AttnView &a, float *sm, const Segment seg, int kvh, int it,
                                          int P, int n_mt, int slot, int n_slots) {
     constexpr int NJ = HD / 8;
-    float *sm_o = sm;                               // [NJ][NW][32] float4
-    float *sm_ml = sm + NW * 32 * NJ * 4;           // [NW][32] float4
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int ms = seg.nrows, group = a.D.nh / a.D.nkv, R = ms * group, qdim = a.D.nh * HD;
     const int n_kl = NW / P;
@@ -211,53 +211,51 @@ __device__ __forceinline__ void tile_end(TileState<HD> &ts, const AttnView &a, f
         __syncthreads();
         return;
     }
-    // layout [column tile][warp][lane]: consecutive lanes write consecutive 16-byte words
+    constexpr int LD = HD + 8;                      // rows of an odd number of 32-byte groups: 8 rows x 4 float2 without bank conflicts
+    float *so = sm;                                 // [NW][16][LD]
+    float *sml = sm + NW * 16 * LD;                 // [NW][16] (max, sum)
 #pragma unroll
-    for (int j = 0; j < NJ; ++j)
-        *reinterpret_cast<float4 *>(sm_o + (size_t)((j * NW + warp) * 32 + lane) * 4) =
-            make_float4(ts.O[j][0], ts.O[j][1], ts.O[j][2], ts.O[j][3]);
-    *reinterpret_cast<float4 *>(sm_ml + (warp * 32 + lane) * 4) = make_float4(ts.m_run[0], ts.l_run[0], ts.m_run[1], ts.l_run[1]);
+    for (int h = 0; h < 2; ++h) {
+        if (!ts.rv[h]) continue;
+        float *dst = so + (warp * 16 + g + 8 * h) * LD + 2 * t;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) *reinterpret_cast<float2 *>(dst + 8 * j) = make_float2(ts.O[j][2 * h], ts.O[j][2 * h + 1]);
+        if (t == 0) *reinterpret_cast<float2 *>(sml + (warp * 16 + g + 8 * h) * 2) = make_float2(ts.m_run[h], ts.l_run[h]);
+    }
     __syncthreads();
-    for (int task = warp; task < P * NJ; task += NW) {
-        const int mp = task / NJ, j = task - mp * NJ;      // query-tile slot of this iteration, column tile
-        const int mt2 = it * P + mp;
-        if (mt2 >= n_mt) continue;
-        float M0 = -INFINITY, M1 = -INFINITY;
+    const int row0 = it * P * 16, n_el = min(R - row0, P * 16) * (HD / 2);
+#pragma unroll 1
+    for (int e = tid; e < n_el; e += NW * 32) {
+        const int rl = e / (HD / 2), col = (e - rl * (HD / 2)) * 2;
+        const int first = (rl >> 4) * 16 + (rl & 15);            // the tile's first warp, its row
+        float M = -INFINITY;
+#pragma unroll 2
+        for (int k2 = 0; k2 < n_kl; ++k2) M = fmaxf(M, sml[(first + k2 * P * 16) * 2]);
+        const float b = M == -INFINITY ? 0.f : M;
+        float L = 0.f, o0 = 0.f, o1 = 0.f;
+#pragma unroll 2
         for (int k2 = 0; k2 < n_kl; ++k2) {
-            const float4 ml = *reinterpret_cast<const float4 *>(sm_ml + ((mp + k2 * P) * 32 + lane) * 4);
-            M0 = fmaxf(M0, ml.x);
-            M1 = fmaxf(M1, ml.z);
+            const int w = first + k2 * P * 16;
+            const float2 ml = *reinterpret_cast<const float2 *>(sml + w * 2);
+            const float2 ov = *reinterpret_cast<const float2 *>(so + w * LD + col);
+            const float f = exp2f(ml.x - b);
+            L += ml.y * f;
+            o0 += ov.x * f;
+            o1 += ov.y * f;
         }
-        const float b0 = M0 == -INFINITY ? 0.f : M0, b1 = M1 == -INFINITY ? 0.f : M1;
-        float L0 = 0.f, L1 = 0.f, o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
-        for (int k2 = 0; k2 < n_kl; ++k2) {
-            const int w2 = mp + k2 * P;
-            const float4 ml = *reinterpret_cast<const float4 *>(sm_ml + (w2 * 32 + lane) * 4);
-            const float f0 = exp2f(ml.x - b0), f1 = exp2f(ml.z - b1);
-            L0 += ml.y * f0;
-            L1 += ml.w * f1;
-            const float4 ov = *reinterpret_cast<const float4 *>(sm_o + (size_t)((j * NW + w2) * 32 + lane) * 4);
-            o0 += ov.x * f0; o1 += ov.y * f0; o2 += ov.z * f1; o3 += ov.w * f1;
-        }
-        const float Mv[2] = {M0, M1}, Lv[2] = {L0, L1}, ov2[2][2] = {{o0, o1}, {o2, o3}};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int r2 = mt2 * 16 + g + 8 * h;
-            if (r2 >= R) continue;
-            int hq, i;
-            split_row(r2, ms, hq, i);
-            const int c = seg.row0 + i, qh = kvh * group + hq;
-            if (n_slots == 1) {
-                const float inv = 1.f / Lv[h];
-                uint32_t hi, lo;
-                split_bf16x2(ov2[h][0] * inv, ov2[h][1] * inv, hi, lo);
-                *reinterpret_cast<uint32_t *>(a.B.ATT + (size_t)c * qdim + qh * HD + 8 * j + 2 * t) = hi;
-                *reinterpret_cast<uint32_t *>(a.B.ATTL + (size_t)c * qdim + qh * HD + 8 * j + 2 * t) = lo;
-            } else {
-                const size_t pi = ((size_t)c * a.D.nh + qh) * n_slots + slot;
-                *reinterpret_cast<float2 *>(a.B.APO + pi * HD + 8 * j + 2 * t) = make_float2(ov2[h][0], ov2[h][1]);
-                if (j == 0 && t == 0) *reinterpret_cast<float2 *>(a.B.APML + pi * 2) = make_float2(Mv[h], Lv[h]);
-            }
+        int hq, i;
+        split_row(row0 + rl, ms, hq, i);
+        const int c = seg.row0 + i, qh = kvh * group + hq;
+        if (n_slots == 1) {
+            const float inv = 1.f / L;
+            uint32_t hi, lo;
+            split_bf16x2(o0 * inv, o1 * inv, hi, lo);
+            *reinterpret_cast<uint32_t *>(a.B.ATT + (size_t)c * qdim + qh * HD + col) = hi;
+            *reinterpret_cast<uint32_t *>(a.B.ATTL + (size_t)c * qdim + qh * HD + col) = lo;
+        } else {
+            const size_t pi = ((size_t)c * a.D.nh + qh) * n_slots + slot;
+            *reinterpret_cast<float2 *>(a.B.APO + pi * HD + col) = make_float2(o0, o1);
+            if (col == 0) *reinterpret_cast<float2 *>(a.B.APML + pi * 2) = make_float2(M, L);
         }
     }
     __syncthreads();
@@ -389,41 +387,46 @@ __device__ __forceinline__ void partial_staged(const AttnView &a, unsigned char 
     const int n_pages = max(p_end - p_begin, 0), n_chunks = (n_pages + CH - 1) / CH;
     const int n_iter = (n_mt + P - 1) / P;          // groups of P concurrent query tiles; each group stages the pages again
 
-    prefetch_weights(*a.pf);
-    pdl_wait();
-    // every thread copies the same pieces of every page: 2*HD 16-byte pieces of keys, 2*HD of values
-    auto issue = [&](int c) {
-        if (c < n_chunks) {
-            unsigned char *buf = smem + (size_t)(c & 1) * CH * S::PAGE;
-            const int p0 = p_begin + c * CH;
-            int pg[CH];
+    // Page ids of the range, one per lane (further ones are read when their chunk is requested).  They are final (the host writes
+    // them before a round's first launch), and so are the pages of positions committed in earlier rounds: their copies go out
+    // before the wait for the producer (8B shape, 4 sequences of 5 rows: 5 us from the wait to the first score, of 40 us per layer
+    // that are not the weight stream).
+    const int ids = lane < n_pages ? pt[p_begin + lane] : 0;
+    const int p_early = min(p_end, a.early_pos >> 4);
+    // every thread copies the same pieces of every page: 2*HD 16-byte pieces of keys, 2*HD of values; pages [from, to) of chunk c
+    auto copy = [&](int c, int from, int to) {
+        const int p0 = p_begin + c * CH;
+#pragma unroll 2
+        for (int p = max(p0, from); p < min(p0 + CH, to); ++p) {
+            const int at = p - p_begin;
+            const int page = at < 32 ? __shfl_sync(0xffffffffu, ids, at) : pt[p];
+            const size_t off = (size_t)page * page_stride + head_off;
+            const unsigned char *kp = reinterpret_cast<const unsigned char *>(a.B.KP + off);
+            const unsigned char *vp = reinterpret_cast<const unsigned char *>(a.B.VP + off);
+            unsigned char *dst = smem + ((size_t)(c & 1) * CH + (p - p0)) * S::PAGE;
 #pragma unroll
-            for (int q = 0; q < CH; ++q) pg[q] = p0 + q < p_end ? pt[p0 + q] : 0;
-#pragma unroll
-            for (int q = 0; q < CH; ++q) {
-                const int p = p0 + q;
-                if (p < p_end) {
-                    const size_t off = (size_t)pg[q] * page_stride + head_off;
-                    const unsigned char *kp = reinterpret_cast<const unsigned char *>(a.B.KP + off);
-                    const unsigned char *vp = reinterpret_cast<const unsigned char *>(a.B.VP + off);
-                    unsigned char *dst = buf + (size_t)q * S::PAGE;
-#pragma unroll
-                    for (int pc = tid; pc < 4 * HD; pc += NW * 32) {
-                        if (pc < 2 * HD) {
-                            const int row = pc / (HD / 8), col = pc - row * (HD / 8);
-                            cp_async16(dst + row * S::KROW + (col ^ ((row & 1) << 2)) * 16, kp + (size_t)pc * 16, true);
-                        } else {
-                            cp_async16(dst + S::KBYTES + (pc - 2 * HD) * 16, vp + (size_t)(pc - 2 * HD) * 16, true);
-                        }
-                    }
+            for (int pc = tid; pc < 4 * HD; pc += NW * 32) {
+                if (pc < 2 * HD) {
+                    const int row = pc / (HD / 8), col = pc - row * (HD / 8);
+                    cp_async16(dst + row * S::KROW + (col ^ ((row & 1) << 2)) * 16, kp + (size_t)pc * 16, true);
+                } else {
+                    cp_async16(dst + S::KBYTES + (pc - 2 * HD) * 16, vp + (size_t)(pc - 2 * HD) * 16, true);
                 }
             }
         }
+    };
+    copy(0, p_begin, p_early);
+    copy(1, p_begin, p_early);
+    prefetch_weights(*a.pf);
+    pdl_wait();
+    auto issue = [&](int c, int from) {
+        if (c < n_chunks) copy(c, from, p_end);
         cp_async_commit();
     };
     for (int it = 0; it < n_iter; ++it) {
-    issue(0);
-    issue(1);
+    // (the early copies belong to the first of these groups)
+    issue(0, it == 0 ? p_early : p_begin);
+    issue(1, it == 0 ? p_early : p_begin);
     const int mt = it * P + warp % P;
     TileState<HD> ts;
     tile_begin<HD>(ts, a, seg, kvh, mt, n_mt, k_hi);
@@ -449,7 +452,7 @@ __device__ __forceinline__ void partial_staged(const AttnView &a, unsigned char 
             }
         }
         __syncthreads();                             // the buffer is free again
-        issue(c + 2);
+        issue(c + 2, p_begin);
     }
     cp_async_wait<0>();
     __syncthreads();                                 // the merge below reuses the staging memory
@@ -459,78 +462,57 @@ __device__ __forceinline__ void partial_staged(const AttnView &a, unsigned char 
 
 // Combines slots 0..n_slots-1 of every (row, head) of a (segment, kv head) in slot order and writes the
 // normalised bf16 result.  The caller has made the slots visible (fence + barrier / arrival counter).
-// NS = compile-time bound on the slots, UE = elements a thread works on at once: the loads of an iteration
-// (UE * NS partial states) are all in flight together.
-template <int HD, int NS, int UE>
+// NS = compile-time bound on the slots: the loads of an element are all in flight together.  Elements go one per thread and
+// iteration, rolled (compact code, see tile_end; with several elements per iteration the merge of 24 rows took 6.7 us).
+template <int HD, int NS>
 __device__ __forceinline__ void merge_slots_n(const AttnView &a, const Segment seg, int kvh, int n_slots) {
     const int ms = seg.nrows, group = a.D.nh / a.D.nkv, R = ms * group, qdim = a.D.nh * HD;
     const int n_el = R * (HD / 4);
-    for (int e0 = threadIdx.x; e0 < n_el; e0 += NW * 32 * UE) {
-        uint2 mlv[UE][NS];
-        uint4 ovv[UE][NS];
-        size_t out_off[UE];
-        bool live[UE];
-        // all loads first, then the arithmetic: two memory latencies per iteration in total
+#pragma unroll 1
+    for (int e = threadIdx.x; e < n_el; e += NW * 32) {
+        const int row = e / (HD / 4), d4 = (e - row * (HD / 4)) * 4;
+        int hq, i;
+        split_row(row, ms, hq, i);
+        const int c = seg.row0 + i, qh = kvh * group + hq;
+        const size_t pi = ((size_t)c * a.D.nh + qh) * n_slots, out_off = (size_t)c * qdim + qh * HD + d4;
+        uint2 mlv[NS];
+        uint4 ovv[NS];
 #pragma unroll
-        for (int u = 0; u < UE; ++u) {
-            const int e = e0 + u * NW * 32;
-            live[u] = e < n_el;
-            const int ee = live[u] ? e : 0;
-            const int row = ee / (HD / 4), d4 = (ee - row * (HD / 4)) * 4;
-            int hq, i;
-            split_row(row, ms, hq, i);
-            const int c = seg.row0 + i, qh = kvh * group + hq;
-            const size_t pi = ((size_t)c * a.D.nh + qh) * n_slots;
-            out_off[u] = (size_t)c * qdim + qh * HD + d4;
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                const int se = s < n_slots ? s : n_slots - 1;       // clamped: unused slots are masked below
-                mlv[u][s] = ldg_act8(a.B.APML + (pi + se) * 2);
-                ovv[u][s] = ldg_act16(a.B.APO + (pi + se) * HD + d4);
-            }
+        for (int s = 0; s < NS; ++s) {
+            const int se = s < n_slots ? s : n_slots - 1;           // clamped: unused slots are masked below
+            mlv[s] = ldg_act8(a.B.APML + (pi + se) * 2);
+            ovv[s] = ldg_act16(a.B.APO + (pi + se) * HD + d4);
         }
+        float M = -INFINITY;
 #pragma unroll
-        for (int u = 0; u < UE; ++u) {
-            float M = -INFINITY;
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                if (s >= n_slots) mlv[u][s].x = 0xff800000u;        // -inf: weight 0
-                M = fmaxf(M, __uint_as_float(mlv[u][s].x));
-            }
-            float l = 0.f, o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                const float f = exp2f(__uint_as_float(mlv[u][s].x) - M);
-                l += f * __uint_as_float(mlv[u][s].y);
-                o0 += f * __uint_as_float(ovv[u][s].x); o1 += f * __uint_as_float(ovv[u][s].y);
-                o2 += f * __uint_as_float(ovv[u][s].z); o3 += f * __uint_as_float(ovv[u][s].w);
-            }
-            const float inv = 1.f / l;
-            uint2 pk, pl;
-            split_bf16x2(o0 * inv, o1 * inv, pk.x, pl.x);
-            split_bf16x2(o2 * inv, o3 * inv, pk.y, pl.y);
-            if (live[u]) {
-                *reinterpret_cast<uint2 *>(a.B.ATT + out_off[u]) = pk;
-                *reinterpret_cast<uint2 *>(a.B.ATTL + out_off[u]) = pl;
-            }
+        for (int s = 0; s < NS; ++s) {
+            if (s >= n_slots) mlv[s].x = 0xff800000u;               // -inf: weight 0
+            M = fmaxf(M, __uint_as_float(mlv[s].x));
         }
+        float l = 0.f, o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            const float f = exp2f(__uint_as_float(mlv[s].x) - M);
+            l += f * __uint_as_float(mlv[s].y);
+            o0 += f * __uint_as_float(ovv[s].x); o1 += f * __uint_as_float(ovv[s].y);
+            o2 += f * __uint_as_float(ovv[s].z); o3 += f * __uint_as_float(ovv[s].w);
+        }
+        const float inv = 1.f / l;
+        uint2 pk, pl;
+        split_bf16x2(o0 * inv, o1 * inv, pk.x, pl.x);
+        split_bf16x2(o2 * inv, o3 * inv, pk.y, pl.y);
+        *reinterpret_cast<uint2 *>(a.B.ATT + out_off) = pk;
+        *reinterpret_cast<uint2 *>(a.B.ATTL + out_off) = pl;
     }
 }
 
 template <int HD>
 __device__ __forceinline__ void merge_slots(const AttnView &a, const Segment seg, int kvh, int n_slots) {
-    // a decode-sized segment has at most one element per thread: one element per thread (least index arithmetic in
-    // front of the loads) and no more loads than the split count needs (1 % of a round against always loading
-    // 16 clamped slots); large segments (prefill passes) batch several elements per thread
-    const int n_el = seg.nrows * (a.D.nh / a.D.nkv) * (HD / 4);
-    if (n_el <= NW * 32) {
-        if (n_slots <= 2) merge_slots_n<HD, 2, 1>(a, seg, kvh, n_slots);
-        else if (n_slots <= 4) merge_slots_n<HD, 4, 1>(a, seg, kvh, n_slots);
-        else if (n_slots <= 8) merge_slots_n<HD, 8, 1>(a, seg, kvh, n_slots);
-        else merge_slots_n<HD, 16, 1>(a, seg, kvh, n_slots);
-    } else if (n_slots > 8) merge_slots_n<HD, 16, 1>(a, seg, kvh, n_slots);
-    else if (n_slots <= 4) merge_slots_n<HD, 4, 4>(a, seg, kvh, n_slots);
-    else merge_slots_n<HD, 8, 2>(a, seg, kvh, n_slots);
+    // no more loads than the split count needs (1 % of a round against always loading 16 clamped slots)
+    if (n_slots <= 2) merge_slots_n<HD, 2>(a, seg, kvh, n_slots);
+    else if (n_slots <= 4) merge_slots_n<HD, 4>(a, seg, kvh, n_slots);
+    else if (n_slots <= 8) merge_slots_n<HD, 8>(a, seg, kvh, n_slots);
+    else merge_slots_n<HD, 16>(a, seg, kvh, n_slots);
 }
 
 }  // namespace attn
