@@ -400,7 +400,8 @@ CtlArgs ctl_base(const del_ctx *c, int plan_idx) {
 // Rows from which on a pass's layer GEMMs run on tcgen05 (rowgemm_tc.cu) rather than register streaming (rowgemm.cu).  The
 // former has a fixed cost of about 14 us per layer (four launches with a ticket and a merge at their end), the latter one
 // that grows with the rows and the weight bytes (and doubles at 33 rows: two launches).  The lines lie where no measured pass
-// is more than 3 % slower than with register streaming.  us per layer, register streaming / tcgen05:
+// is more than 3 % slower than with register streaming.  us per layer, register streaming / tcgen05 (before the weights were
+// marked evict-first in L2, which took 1 to 5 % off both):
 //   13B shape (635 MB)   4 rows 126 / 131,   5: 138 / 131,   8: 148 / 132,   13: 219 / 137
 //   570 MB               4 rows 116 / 121,   5: 130 / 122,   8: 137 / 123,    9: 189 / 131
 //   510 MB               5 rows 105 / 111,   8: 115 / 113,   9: 149 / 117,   16: 171 / 118
