@@ -338,8 +338,14 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
         if (lane == 0) {
             // With up to two row tiles the weights are most of what a launch reads, each tile at about the same time by both: it goes
             // first from L2, and activations and code stay.  ms per prompt, 7B shape: 45 positions 5.97 -> 5.40, 100: 6.18 -> 5.66,
-            // 200: 8.28 -> 8.00; 1B, 45: 2.01 -> 1.90.  With more row tiles (512 to 3072 positions) it changes nothing or costs 1 %.
-            const uint64_t pol = n_mt <= 2 ? l2_evict_first() : l2_evict_normal();
+            // 200: 8.28 -> 8.00; 1B, 45: 2.01 -> 1.90.  With more row tiles (512 to 3072 positions) it changes nothing or costs 1 %, and so
+            // does a load with the normal policy given explicitly: those load without one.
+            const bool few = n_mt <= 2;
+            const uint64_t pol = l2_evict_first();
+            auto load_w = [&](void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
+                if (few) tma_load_2d(dst, map, x, y, bar, pol);
+                else tma_load_2d(dst, map, x, y, bar);
+            };
             const int n_qt = (p.D.nh * p.D.hd + bn - 1) / bn, n_kt = (p.D.nkv * p.D.hd + bn - 1) / bn;
             int s = 0;
             uint32_t phase = 1;
@@ -361,11 +367,11 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
                     if (EPI == PF_GATEUP) {
                         // accumulator columns 0 .. bn/2 - 1: gate rows of this tile, bn/2 .. bn - 1: the same rows of W_up
                         for (int r = 0; r < bn / 2; r += 64) {
-                            tma_load_2d(sb + r * 128, &maps.b0, kb * BK, nt * (bn / 2) + r, &full_bar[s], pol);
-                            tma_load_2d(sb + (bn / 2 + r) * 128, &maps.b1, kb * BK, nt * (bn / 2) + r, &full_bar[s], pol);
+                            load_w(sb + r * 128, &maps.b0, kb * BK, nt * (bn / 2) + r, &full_bar[s]);
+                            load_w(sb + (bn / 2 + r) * 128, &maps.b1, kb * BK, nt * (bn / 2) + r, &full_bar[s]);
                         }
                     } else {
-                        for (int r = 0; r < bn; r += 128) tma_load_2d(sb + r * 128, mb, kb * BK, y + r, &full_bar[s], pol);
+                        for (int r = 0; r < bn; r += 128) load_w(sb + r * 128, mb, kb * BK, y + r, &full_bar[s]);
                     }
                     if (++s == n_stages) { s = 0; phase ^= 1; }
                 }
