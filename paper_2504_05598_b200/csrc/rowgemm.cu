@@ -94,10 +94,18 @@ __global__ void __launch_bounds__(NW * 32, (NW == 8 && NT <= 4 ? 2 : 1)) rowgemm
     const int nkw = (n_ksteps + NW - 1) / NW;       // k-steps per warp and tile (the last ones may be empty)
     __shared__ int s_claim[2];                      // tile claimed for the turn after next (double-buffered)
 
-    // The weights pass through L2 once.  Marked as the first to go, they leave the lines that every launch needs again: its code
-    // (a layer streams 405 MB at the 7B shape between two runs of the same epilogue), activations, page tables.  ms per plain
-    // round, 7B shape 2.520 -> 2.498, 1B 0.680 -> 0.669; 13B, 5 rows at 2 500 positions 8.85 -> 8.57.
-    const uint64_t pol = l2_evict_first();
+    // Marked as the first to go from L2, the weights leave the lines that every launch needs again: its code (a layer streams 405 MB
+    // at the 7B shape between two runs of the same epilogue), activations, page tables.  ms per plain round, 7B shape 2.520 -> 2.498,
+    // 1B 0.680 -> 0.669.  A pass of more than 32 rows reads them again in its second launch, and gains all the same (50 MB per
+    // layer, rounds with 48-row passes 2.267 -> 2.228, 64 rows 2.810 -> 2.770).  Not in the one-row head: the policy's register is
+    // one too many there (12 bytes of spills), and without it rounds with a head every two layers take the same time (1B shape, six
+    // drafts at layer 2: 1.742 -> 1.741; 7B, four: 3.744 -> 3.743).
+    constexpr bool EVICT_FIRST = !(EPI == EPI_LMHEAD && NT == 1);
+    const uint64_t pol = EVICT_FIRST ? l2_evict_first() : 0;
+    auto load_stream = [&](const bf16 *p, bool ok) {
+        if constexpr (EVICT_FIRST) return ldg_stream16_pred(p, ok, pol);
+        else return ldg_stream16_pred(p, ok);
+    };
     uint4 wa[U], wb[U];
     uint4 xv[U][NT];
     const bf16 *xrow[NT];
@@ -115,8 +123,8 @@ __global__ void __launch_bounds__(NW * 32, (NW == 8 && NT <= 4 ? 2 : 1)) rowgemm
         for (int u = 0; u < U; ++u) {
             const int k0 = (warp + NW * (u0 + u)) << 5;
             const bool ok = live && (u0 + u < nkw) && (k0 + 8 * t < K);
-            wa[u] = ldg_stream16_pred(base + k0, ok, pol);
-            wb[u] = ldg_stream16_pred(base_hi + k0, ok, pol);
+            wa[u] = load_stream(base + k0, ok);
+            wb[u] = load_stream(base_hi + k0, ok);
         }
     };
     auto load_x = [&](int u0, bool live) {
