@@ -150,9 +150,10 @@ __device__ __forceinline__ void page_update(TileState<HD> &ts, const uint4 (&kf)
 
 // The warps of each query tile merge their states through shared memory and the result is written: normalised to ATT when
 // n_slots == 1, otherwise as a partial state to slot `slot`.  it = iteration over groups of P concurrent query tiles.
-// The code for more than 8 rows has rolled loops: it runs once per launch, and fetching its instructions costs more than
-// executing them (the weight stream of a layer evicts them from L2).  Four sequences of 4 + 1 rows, 8B shape: 7.13 -> 6.93 ms
-// per round together with merge_slots.
+// The code for more than 8 rows has rolled loops over four columns per thread: it runs once per launch, and what unrolling gains is
+// lost again on fetching the instructions.  us per layer, passes of one sequence, fully unrolled / rolled, two columns per thread /
+// rolled, four: 8B shape, 8 rows 102.5 / 103.2 / 101.3, 32 rows 279.6 / 279.6 / 273.5; 1B 8 rows 46.9 / 46.7 / 45.6, 32 rows
+// 109.2 / 108.8 / 105.9; 7B 16 rows 139.8 / 139.6 / 138.2.
 template <int HD>
 __device__ __forceinline__ void tile_end(TileState<HD> &ts, const AttnView &a, float *sm, const Segment seg, int kvh, int it,
                                          int P, int n_mt, int slot, int n_slots) {
@@ -223,38 +224,38 @@ __device__ __forceinline__ void tile_end(TileState<HD> &ts, const AttnView &a, f
         if (t == 0) *reinterpret_cast<float2 *>(sml + (warp * 16 + g + 8 * h) * 2) = make_float2(ts.m_run[h], ts.l_run[h]);
     }
     __syncthreads();
-    const int row0 = it * P * 16, n_el = min(R - row0, P * 16) * (HD / 2);
+    const int row0 = it * P * 16, n_el = min(R - row0, P * 16) * (HD / 4);
 #pragma unroll 1
     for (int e = tid; e < n_el; e += NW * 32) {
-        const int rl = e / (HD / 2), col = (e - rl * (HD / 2)) * 2;
-        const int first = (rl >> 4) * 16 + (rl & 15);            // the tile's first warp, its row
+        const int rl = e / (HD / 4), col = (e - rl * (HD / 4)) * 4;     // rl: row of the P tiles; its first warp's row in `so` as well
         float M = -INFINITY;
 #pragma unroll 2
-        for (int k2 = 0; k2 < n_kl; ++k2) M = fmaxf(M, sml[(first + k2 * P * 16) * 2]);
+        for (int k2 = 0; k2 < n_kl; ++k2) M = fmaxf(M, sml[(rl + k2 * P * 16) * 2]);
         const float b = M == -INFINITY ? 0.f : M;
-        float L = 0.f, o0 = 0.f, o1 = 0.f;
+        float L = 0.f;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 2
         for (int k2 = 0; k2 < n_kl; ++k2) {
-            const int w = first + k2 * P * 16;
+            const int w = rl + k2 * P * 16;
             const float2 ml = *reinterpret_cast<const float2 *>(sml + w * 2);
-            const float2 ov = *reinterpret_cast<const float2 *>(so + w * LD + col);
+            const float4 ov = *reinterpret_cast<const float4 *>(so + w * LD + col);
             const float f = exp2f(ml.x - b);
             L += ml.y * f;
-            o0 += ov.x * f;
-            o1 += ov.y * f;
+            o.x += ov.x * f; o.y += ov.y * f; o.z += ov.z * f; o.w += ov.w * f;
         }
         int hq, i;
         split_row(row0 + rl, ms, hq, i);
         const int c = seg.row0 + i, qh = kvh * group + hq;
         if (n_slots == 1) {
             const float inv = 1.f / L;
-            uint32_t hi, lo;
-            split_bf16x2(o0 * inv, o1 * inv, hi, lo);
-            *reinterpret_cast<uint32_t *>(a.B.ATT + (size_t)c * qdim + qh * HD + col) = hi;
-            *reinterpret_cast<uint32_t *>(a.B.ATTL + (size_t)c * qdim + qh * HD + col) = lo;
+            uint2 hi, lo;
+            split_bf16x2(o.x * inv, o.y * inv, hi.x, lo.x);
+            split_bf16x2(o.z * inv, o.w * inv, hi.y, lo.y);
+            *reinterpret_cast<uint2 *>(a.B.ATT + (size_t)c * qdim + qh * HD + col) = hi;
+            *reinterpret_cast<uint2 *>(a.B.ATTL + (size_t)c * qdim + qh * HD + col) = lo;
         } else {
             const size_t pi = ((size_t)c * a.D.nh + qh) * n_slots + slot;
-            *reinterpret_cast<float2 *>(a.B.APO + pi * HD + col) = make_float2(o0, o1);
+            *reinterpret_cast<float4 *>(a.B.APO + pi * HD + col) = o;
             if (col == 0) *reinterpret_cast<float2 *>(a.B.APML + pi * 2) = make_float2(M, L);
         }
     }
