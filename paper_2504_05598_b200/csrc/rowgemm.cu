@@ -97,10 +97,10 @@ __global__ void __launch_bounds__(NW * 32, (NW == 8 && NT <= 4 ? 2 : 1)) rowgemm
     // Marked as the first to go from L2, the weights leave the lines that every launch needs again: its code (a layer streams 405 MB
     // at the 7B shape between two runs of the same epilogue), activations, page tables.  ms per plain round, 7B shape 2.520 -> 2.498,
     // 1B 0.680 -> 0.669.  A pass of more than 32 rows reads them again in its second launch, and gains all the same (50 MB per
-    // layer, rounds with 48-row passes 2.267 -> 2.228, 64 rows 2.810 -> 2.770).  Not in the one-row head: the policy's register is
-    // one too many there (12 bytes of spills), and without it rounds with a head every two layers take the same time (1B shape, six
-    // drafts at layer 2: 1.742 -> 1.741; 7B, four: 3.744 -> 3.743).
-    constexpr bool EVICT_FIRST = !(EPI == EPI_LMHEAD && NT == 1);
+    // layer, rounds with 48-row passes 2.267 -> 2.228, 64 rows 2.810 -> 2.770).  The head goes without: one launch reads nothing again,
+    // and at its one-row variant's register cap the policy is a value too many (12 bytes of spills).  us alone without / with, 1B
+    // shape: 1 row 88.6 / 89.7, 64 rows 366.4 / 369.5; 8B 167.1 / 167.9, 64 rows 593.5 / 596.0.  Rounds with a head every two layers tie.
+    constexpr bool EVICT_FIRST = EPI != EPI_LMHEAD;
     const uint64_t pol = EVICT_FIRST ? l2_evict_first() : 0;
     auto load_stream = [&](const bf16 *p, bool ok) {
         if constexpr (EVICT_FIRST) return ldg_stream16_pred(p, ok, pol);
