@@ -389,8 +389,8 @@ __device__ __forceinline__ void partial_staged(const AttnView &a, unsigned char 
     const int n_iter = (n_mt + P - 1) / P;          // groups of P concurrent query tiles; each group stages the pages again
 
     // Page ids and the pages of positions committed in earlier rounds are final (the host writes the ids before a round's first
-    // launch): the copies of such pages go out before the wait for the producer (8B shape, 4 sequences of 5 rows: 5 us from the wait
-    // to the first score, of 40 us per layer that are not the weight stream).
+    // launch): the copies of such pages go out before the wait for the producer.  ms per round without / with them: 1B shape, 8 sequences
+    // of 6 rows at 2 000 positions 3.509 / 3.471, 4 at 1 000 2.415 / 2.400; 8B shape 0 to 0.8 %, within the spread.
     // The ids are read ahead, one per lane, a window of whole chunks at a time: `ids` is the window the copies are in, `ids_next` the
     // one behind it, requested when they enter `ids`.  (With one load per page behind the 32nd, in front of that page's copies, rounds
     // whose ranges have 60 to 80 pages took 1 % longer: 1B shape, 8 sequences of 6 rows at 2 000 positions 3.506 against 3.470 ms,
@@ -444,7 +444,10 @@ __device__ __forceinline__ void partial_staged(const AttnView &a, unsigned char 
     TileState<HD> ts;
     tile_begin<HD>(ts, a, seg, kvh, mt, n_mt, k_hi);
     for (int c = 0; c < n_chunks; ++c) {
-        cp_async_wait<1>();                          // chunk c has landed (chunk c + 1 may be in flight)
+        // chunk c has landed; chunk c + 1 may be in flight, but for the committed pages of the second chunk, which were requested with
+        // the first's (a group of their own gained nothing: 8B shape, 4 sequences of 4 and 5 rows 5.339 and 6.258 ms, with it 5.308
+        // and 6.292)
+        cp_async_wait<1>();
         __syncthreads();
         const unsigned char *buf = smem + (size_t)(c & 1) * CH * S::PAGE;
         if (mt < n_mt) {
@@ -476,7 +479,8 @@ __device__ __forceinline__ void partial_staged(const AttnView &a, unsigned char 
 // Combines slots 0..n_slots-1 of every (row, head) of a (segment, kv head) in slot order and writes the
 // normalised bf16 result.  The caller has made the slots visible (fence + barrier / arrival counter).
 // NS = compile-time bound on the slots: the loads of an element are all in flight together.  Elements go one per thread and
-// iteration, rolled (compact code, see tile_end; with several elements per iteration the merge of 24 rows took 6.7 us).
+// iteration, rolled: ms per round, batched and unrolled / this, 1B shape, 8 sequences of 6 rows at 2 000 positions 3.496 / 3.471, 4 at
+// 1 000 2.426 / 2.400, 8B, 4 of 4 rows at 1 024 5.315 / 5.268.
 template <int HD, int NS>
 __device__ __forceinline__ void merge_slots_n(const AttnView &a, const Segment seg, int kvh, int n_slots) {
     const int ms = seg.nrows, group = a.D.nh / a.D.nkv, R = ms * group, qdim = a.D.nh * HD;

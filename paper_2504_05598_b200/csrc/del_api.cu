@@ -398,21 +398,22 @@ CtlArgs ctl_base(const del_ctx *c, int plan_idx) {
 }
 
 // Rows from which on a pass's layer GEMMs run on tcgen05 (rowgemm_tc.cu) rather than register streaming (rowgemm.cu).  The
-// former has a fixed cost of about 14 us per layer (four launches with a ticket and a merge at their end), the latter one
-// that grows with the rows and the weight bytes (and doubles at 33 rows: two launches).  The lines lie where no measured pass
-// is more than 3 % slower than with register streaming.  us per layer, register streaming / tcgen05 (before the weights were
-// marked evict-first in L2, which took 1 to 5 % off both):
-//   13B shape (635 MB)   4 rows 126 / 131,   5: 138 / 131,   8: 148 / 132,   13: 219 / 137
-//   570 MB               4 rows 116 / 121,   5: 130 / 122,   8: 137 / 123,    9: 189 / 131
-//   510 MB               5 rows 105 / 111,   8: 115 / 113,   9: 149 / 117,   16: 171 / 118
-//   8B shape (436 MB)    5 rows  99 / 101,   8: 106 / 104,   9: 138 / 105,   16: 158 / 110,   32: 280 / 132
-//   7B shape (405 MB)    5 rows  89 /  95,   8:  93 /  98,   9: 126 / 102,   16: 141 / 102,   32: 258 / 124
-//   1B shape (122 MB)    8 rows  47 /  60,   9:  64 /  63,  16:  73 /  64,   32: 110 /  89
-//   88 MB                9 rows  59 /  61,  16:  69 /  65,  17:  86 /  82,   32: 105 /  92
-//   78 MB               16 rows  58 /  58,  17:  75 /  76,  32:  87 /  86,   33: 112 /  98
-//   67 MB               17 rows  75 /  82,  32:  94 / 100,  33: 118 / 112,   64: 186 / 172
-//   50 MB               32 rows  72 /  81,  33:  91 /  93,  48: 119 / 104,   64: 137 / 140
-//   tiny (1.6 MB)        8 rows  17 /  34,  16:  24 /  36,  32:  33 /  52
+// former has a fixed cost per layer (four launches with a ticket and a merge at their end: 20 us at the 1B shape, 12 at 7B, 2 at 13B),
+// the latter one that grows with the rows and the weight bytes (and doubles at 33 rows: two launches).  The lines lie where no
+// measured pass is more than 3 % slower than with register streaming.  us per layer, register streaming / tcgen05, both with the
+// weights marked evict-first in L2 (which took 0 to 2 % off the former and 2 to 13 % off the latter: from 6 rows at 400 MB and 5 at
+// 510 MB the latter is ahead by now, 8B shape, 8 rows 106 / 97; the lines are the ones drawn before that):
+//   13B shape (635 MB)   4 rows 123 / 123,   5: 144 / 123,   8: 156 / 124,   13: 222 / 128
+//   570 MB               4 rows 112 / 112,   5: 130 / 112,   8: 141 / 114,    9: 190 / 116
+//   510 MB               5 rows 108 / 106,   8: 114 / 106,   9: 151 / 106,   16: 175 / 109
+//   8B shape (436 MB)    5 rows  97 /  95,   8: 106 /  97,   9: 137 /  98,   16: 157 / 102,   32: 280 / 124
+//   7B shape (405 MB)    5 rows  88 /  90,   8:  94 /  91,   9: 124 /  93,   16: 141 /  95,   32: 258 / 112
+//   1B shape (122 MB)    8 rows  46 /  56,   9:  63 /  60,  16:  72 /  62,   32: 109 /  86
+//   88 MB                9 rows  58 /  59,  16:  68 /  62,  17:  85 /  78,   32: 105 /  92
+//   78 MB               16 rows  57 /  55,  17:  72 /  73,  32:  86 /  83,   33: 108 /  95
+//   67 MB               17 rows  73 /  81,  32:  93 /  99,  33: 116 / 112,   64: 182 / 170
+//   50 MB               32 rows  71 /  81,  33:  88 /  93,  48: 116 / 104,   64: 135 / 138
+//   tiny (1.6 MB)        8 rows  16 /  34,  16:  23 /  37,  32:  32 /  52
 int rows_min_tc(const Dims &D) {
     const double mb = 2e-6 * ((double)D.d * (D.nh + 2 * D.nkv) * D.hd + (double)D.nh * D.hd * D.d + 3.0 * D.d * D.F);
     return mb >= 550 ? 5 : mb >= 100 ? 9 : mb >= 80 ? 17 : mb >= 64 ? 33 : DEL_ROWS_MAX + 1;
@@ -1250,9 +1251,10 @@ int del_prefill(del_ctx *c, int sq, const int32_t *prompt, int n_prompt, int max
     // in slots 0..W-1 of the stack
     std::vector<std::pair<int, int>> chunks;
     // Prompts longer than the longest window go through the tensor-core prefill as a whole: the decode kernels would take two
-    // passes (the window is one of its own) where a window alone takes one, which is faster.  us per layer, decode kernels /
-    // prefill kernels: 13B shape 33 positions 304 / 234, 77: 369 / 244; 7B 33: 221 / 204, 48: 248 / 205, 77: 289 / 210;
-    // 1B 33: 142 / 130, 48: 172 / 131; 88 MB per layer 33: 136 / 113; 24 MB 33: 80 / 73; tiny 33: 59 / 48, 77: 93 / 54.
+    // passes (the window is one of its own) where a window alone takes one, which is faster.  ms per prompt, decode kernels /
+    // prefill kernels: 13B shape 33 positions 11.13 / 8.35, 77: 13.33 / 9.34; 8B 33: 7.44 / 5.97; 7B 33: 6.17 / 5.38, 48: 6.79 / 5.45,
+    // 77: 7.85 / 5.72; 1B 33: 2.13 / 1.90, 48: 2.60 / 1.92; 16 layers of 88 MB 33: 2.10 / 1.68, of 24 MB 33: 1.27 / 1.17; tiny 33:
+    // 0.242 / 0.223, 77: 0.393 / 0.246.
     if (c->pf_ok && !(c->flags & FLAG_NO_BULK_PREFILL) && n_prompt > WINDOW_MAX) {
         rc = prefill_bulk(c, sq, n_prompt, n_prompt - W);
         if (rc) return rc;

@@ -337,9 +337,11 @@ __global__ void __launch_bounds__(PF_THREADS, 1) prefill_gemm_kernel(const __gri
     if (warp == 0) {
         if (lane == 0) {
             // With up to two row tiles the weights are most of what a launch reads, each tile at about the same time by both: it goes
-            // first from L2, and activations and code stay.  ms per prompt, 7B shape: 45 positions 5.97 -> 5.40, 100: 6.18 -> 5.66,
-            // 200: 8.28 -> 8.00; 1B, 45: 2.01 -> 1.90.  With more row tiles (512 to 3072 positions) it changes nothing or costs 1 %, and so
-            // does a load with the normal policy given explicitly: those load without one.
+            // first from L2, and activations and code stay.  ms per prompt without / with, 7B shape: 45 positions 6.01 / 5.44, 128:
+            // 6.38 / 5.97, 160: 8.98 / 8.82, 256: 9.44 / 9.27; 1B 45: 2.01 / 1.92, 256: 2.42 / 2.35; 8B and 13B 1 to 7 % less; tiny (all
+            // weights stay in L2 anyway) 0 to 1 % more.  With more row tiles (tried up to four) 257 to 384 positions would gain 2 % at the 1B shape, 1 % at
+            // 7B and 0 to 1.5 % at 8B and 13B, 385 to 512 -1 to 2 %, longer ones nothing or -1 %; a load with the normal policy given
+            // explicitly costs the latter too.  Those load without one.
             const bool few = n_mt <= 2;
             const uint64_t pol = l2_evict_first();
             auto load_w = [&](void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
@@ -537,13 +539,15 @@ int n_tiles_of(int epi, const Dims &D, int bn) {
 // Tile width and parts of K of a launch: the choice with the smallest estimated time, waves of tiles on the SMs x (K blocks of
 // a tile x what a block takes) + the last tile's epilogue + the merge of the parts.  The constants are microseconds fitted to 897
 // launches of six layer shapes (50 to 635 MB) at 48 to 2048 rows: 6 % rms, and no launch whose choice is more than 7 % slower
-// than the best of the five.  Measured, us, 256 wide / 128 wide / 128 wide with K in 2, 3, 4 parts:
-//   7B shape,   48 rows: QKV 50 / 35,  O 49 / 34 / 30, 29, 29,  gate/up 53 / 64,  down 113 / 77 / 53, 44, 42
-//   7B shape,  160 rows: QKV 55 / 61,  O 53 / 36 / 34,          gate/up 92 / 90,  down 115 / 79 / 57
-//   7B shape,  512 rows: QKV 89 / 92,  O 54 / 39,               gate/up 137 / 154, down 118 / 87
+// than the best of the five.  That holds for launches of up to two row tiles with their weights marked evict-first, too: seven shapes
+// at 48 to 512 rows measured again, choices at most 4 % from the best.  Measured, us, 256 wide / 128 wide / 128 wide with K
+// in 2, 3, 4 parts (1024 rows: before that):
+//   7B shape,   48 rows: QKV 49 / 35,  O 48 / 34 / 30, 29, 29,  gate/up 53 / 66,  down 112 / 78 / 52, 44, 41
+//   7B shape,  160 rows: QKV 54 / 60,  O 53 / 36 / 33,          gate/up 90 / 91,  down 114 / 78 / 56
+//   7B shape,  512 rows: QKV 89 / 92,  O 54 / 39,               gate/up 137 / 153, down 118 / 85
 //   7B shape, 1024 rows: QKV 142 / 188, O 59 / 71,              gate/up 232 / 315, down 134 / 169
 //   13B shape, 1024 rows: QKV 223 / 272, O 119 / 123,           gate/up 352 / 471, down 308 / 312
-//   1B shape,  160 rows: QKV 32 / 22 / 25, 26,  O 34 / 23 / 26, 26, 28,  gate/up 32 / 38,  down 90 / 61 / 45, 40, 38
+//   1B shape,  160 rows: QKV 31 / 22 / 24, 26,  O 34 / 23 / 25, 26, 27,  gate/up 32 / 37,  down 88 / 60 / 44, 39, 38
 // (a merge costs as much as 25 to 40 K blocks, so K of 2048 is not cut)
 struct Split { int bn, parts; double us; };
 Split choose_split(int epi, const Dims &D, int M, int n_sms) {

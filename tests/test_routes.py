@@ -10,58 +10,58 @@ CONFIGS = dict(synth.CONFIGS, mid=MID)
 
 # us per launch of the prefill GEMMs: tiles 256 wide, 128 wide, 128 wide with K in 2, 3, 4 parts
 LAUNCHES = """
-mid              48 qkv        22.7   16.4   20.0   21.1   22.7
-mid              48 o          23.9   16.8   20.6   21.9   23.0
-mid              48 gate_up    23.3   17.0   22.0
-mid              48 down       48.2   33.4   29.4   28.3   28.0
-mid             512 qkv        28.2   19.9
-mid             512 o          30.2   20.2   24.6   26.0
-mid             512 gate_up    26.6   29.9
-mid             512 down       54.0   36.5   33.4   32.5
-llama32_1b       48 qkv        30.1   20.7   23.1   23.9   24.9
-llama32_1b       48 o          30.4   20.6   23.6   24.1   24.7
-llama32_1b       48 gate_up    32.2   23.2
-llama32_1b       48 down       92.5   61.4   44.5   38.5   35.7
-llama32_1b      160 qkv        32.0   22.3   25.1   26.0
-llama32_1b      160 o          33.9   22.8   25.8   26.4   27.7
-llama32_1b      160 gate_up    32.4   37.5
-llama32_1b      160 down       89.6   60.8   45.2   40.1   38.3
-llama32_1b      512 qkv        32.6   23.2
-llama32_1b      512 o          34.1   23.1   26.5
-llama32_1b      512 gate_up    54.8   66.8
-llama32_1b      512 down       90.8   63.0   47.7
+mid              48 qkv        22.4   16.1   20.0   21.0   22.5
+mid              48 o          23.6   16.7   20.7   22.1   23.4
+mid              48 gate_up    23.6   16.8   22.3
+mid              48 down       47.6   33.0   29.0   28.1   27.9
+mid             512 qkv        28.1   19.8
+mid             512 o          30.4   20.1   24.7   26.1
+mid             512 gate_up    26.9   30.1
+mid             512 down       54.5   36.6   33.7   32.9
+llama32_1b       48 qkv        26.8   19.2   21.5   22.1   23.7
+llama32_1b       48 o          27.6   19.6   22.2   23.0   23.9
+llama32_1b       48 gate_up    29.7   22.2
+llama32_1b       48 down       83.4   57.8   41.5   35.9   34.0
+llama32_1b      160 qkv        31.4   21.6   24.1   25.6
+llama32_1b      160 o          33.9   22.7   25.3   26.1   27.4
+llama32_1b      160 gate_up    32.0   36.8
+llama32_1b      160 down       88.2   60.3   44.4   39.1   37.6
+llama32_1b      512 qkv        32.5   23.2
+llama32_1b      512 o          34.5   23.0   26.7
+llama32_1b      512 gate_up    54.7   66.3
+llama32_1b      512 down       90.2   62.4   48.1
 llama32_1b     1024 qkv        33.8   36.8
 llama32_1b     1024 o          34.9   24.2
 llama32_1b     1024 gate_up    96.2  110.8
 llama32_1b     1024 down       92.2   67.4
-llama2_7b        48 qkv        49.5   35.2
-llama2_7b        48 o          49.0   33.5   30.1   29.0   29.3
-llama2_7b        48 gate_up    53.0   63.7
-llama2_7b        48 down      112.9   76.9   52.5   44.4   41.5
-llama2_7b       160 qkv        55.3   61.1
-llama2_7b       160 o          53.3   36.1   33.7
-llama2_7b       160 gate_up    91.5   90.3
-llama2_7b       160 down      115.4   79.3   56.6
-llama2_7b       512 qkv        88.8   92.2
-llama2_7b       512 o          53.8   39.2
-llama2_7b       512 gate_up   136.8  153.8
-llama2_7b       512 down      117.9   87.2
+llama2_7b        48 qkv        49.1   35.2
+llama2_7b        48 o          48.1   33.7   29.6   28.6   28.8
+llama2_7b        48 gate_up    53.2   65.8
+llama2_7b        48 down      112.4   78.3   51.7   43.5   40.6
+llama2_7b       160 qkv        54.1   60.3
+llama2_7b       160 o          53.3   35.7   33.1
+llama2_7b       160 gate_up    90.4   90.8
+llama2_7b       160 down      114.2   78.2   55.7
+llama2_7b       512 qkv        88.9   92.2
+llama2_7b       512 o          53.9   38.8
+llama2_7b       512 gate_up   137.1  153.0
+llama2_7b       512 down      117.9   85.0
 llama2_7b      1024 qkv       141.7  187.7
 llama2_7b      1024 o          59.4   70.6
 llama2_7b      1024 gate_up   232.1  315.1
 llama2_7b      1024 down      134.1  169.2
-llama3_8b_b4    160 qkv        51.4   36.2
-llama3_8b_b4    160 o          53.8   36.4   33.6
-llama3_8b_b4    160 gate_up    95.0  118.9
-llama3_8b_b4    160 down      145.0   99.2   67.0
+llama3_8b_b4    160 qkv        51.0   35.4
+llama3_8b_b4    160 o          53.2   35.8   32.8
+llama3_8b_b4    160 gate_up    94.5  119.1
+llama3_8b_b4    160 down      144.3   99.2   66.0
 llama3_8b_b4   2048 qkv       147.9  192.3
 llama3_8b_b4   2048 o         105.3  133.1
 llama3_8b_b4   2048 gate_up   615.3  785.9
 llama3_8b_b4   2048 down      331.8  434.8
-llama2_13b      160 qkv        67.7   75.6
-llama2_13b      160 o          64.5   43.5
-llama2_13b      160 gate_up   114.7  112.4
-llama2_13b      160 down      142.4   97.8
+llama2_13b      160 qkv        67.0   77.6
+llama2_13b      160 o          64.0   42.8
+llama2_13b      160 gate_up   113.9  113.0
+llama2_13b      160 down      141.5   97.5
 llama2_13b     1024 qkv       223.3  272.3
 llama2_13b     1024 o         118.6  122.9
 llama2_13b     1024 gate_up   351.8  471.2
@@ -85,17 +85,17 @@ def test_prefill_tiles_are_near_the_best_measured(line):
 
 # d_model, heads, kv heads, head dimension, d_ffn; then us per layer of a pass of so many rows: register streaming / tcgen05
 PASSES = """
-1536,24,8,64,4096        4:28/46 5:32/45 8:34/47 9:45/52 16:50/53 17:59/71 24:66/76 32:72/81 33:91/93 48:119/104 64:137/140
-1792,28,4,64,4864        4:32/51 5:37/51 8:39/53 9:52/59 16:62/63 17:75/82 24:83/87 32:94/100 33:118/112 48:157/129 64:186/172
-2048,32,8,64,4608        4:32/50 5:37/51 8:40/53 9:52/56 16:58/58 17:75/76 24:79/81 32:87/86 33:112/98 48:140/107 64:168/144
-2048,32,4,64,5632        4:34/53 5:40/53 8:43/55 9:59/61 16:69/65 17:86/82 24:93/84 32:105/93 33:133/109 48:171/122 64:208/165
-2048,32,8,64,8192        4:36/59 5:44/58 8:47/60 9:64/64 16:73/64 17:94/81 24:100/85 32:110/90 33:141/103 48:180/111 64:216/145
-4096,32,32,128,11008     4:83/96 5:89/95 8:93/98 9:126/102 16:141/102 17:224/116 24:236/118 32:258/124 33:327/137 48:393/141 64:508/162
-4096,32,8,128,14336      4:88/103 5:99/101 8:106/104 9:138/105 16:158/110 17:245/124 24:256/126 32:280/132 33:359/148 48:432/156 64:561/187
-4608,36,36,128,12288     4:99/111 5:105/111 8:115/113 9:149/117 16:171/118 17:244/132 24:262/134 32:285/139 33:372/152 48:450/155 64:564/173
-4864,38,38,128,13056     4:116/121 5:130/122 8:137/123 9:189/131 16:214/130 17:315/142 24:332/145 32:361/148 33:470/165 48:573/170 64:715/187
-5120,40,40,128,13824     4:126/131 5:140/132 8:148/132 9:205/138 16:234/139 17:329/154 24:348/155 32:378/161 33:493/176 48:606/179 64:746/201
-256,4,4,64,688           4:18/33 5:17/33 8:17/34 9:23/36 16:24/36 17:30/50 24:31/50 32:33/52 33:49/63 48:54/66 64:58/79
+1536,24,8,64,4096        4:27/44 5:31/44 8:33/46 9:43/51 16:48/52 17:58/70 24:64/74 32:71/81 33:88/93 48:116/104 64:135/138
+1792,28,4,64,4864        4:32/50 5:36/50 8:38/52 9:51/57 16:61/62 17:73/81 24:82/88 32:93/99 33:116/112 48:153/130 64:182/170
+2048,32,8,64,4608        4:31/47 5:35/48 8:39/50 9:49/53 16:57/55 17:72/73 24:78/77 32:86/83 33:108/95 48:136/104 64:166/143
+2048,32,4,64,5632        4:35/51 5:39/51 8:43/53 9:58/59 16:68/62 17:85/78 24:93/82 32:105/92 33:130/107 48:168/121 64:207/164
+2048,32,8,64,8192        4:36/54 5:45/55 8:46/57 9:63/60 16:72/62 17:93/77 24:99/80 32:109/86 33:136/98 48:176/104 64:214/136
+4096,32,32,128,11008     4:81/88 5:88/90 8:94/91 9:124/93 16:141/95 17:223/105 24:235/107 32:258/112 33:324/122 48:392/127 64:509/148
+4096,32,8,128,14336      4:88/93 5:97/95 8:106/97 9:137/98 16:157/102 17:242/113 24:256/117 32:280/124 33:355/138 48:432/149 64:561/183
+4608,36,36,128,12288     4:97/102 5:108/106 8:114/106 9:151/106 16:175/109 17:244/119 24:260/122 32:286/128 33:373/137 48:456/142 64:565/169
+4864,38,38,128,13056     4:112/112 5:130/112 8:141/114 9:190/116 16:220/119 17:315/129 24:334/132 32:365/139 33:468/147 48:575/153 64:718/178
+5120,40,40,128,13824     4:123/123 5:144/123 8:156/124 9:208/125 16:240/128 17:330/142 24:350/143 32:382/151 33:490/164 48:605/169 64:750/197
+256,4,4,64,688           4:17/33 5:17/34 8:16/34 9:23/37 16:23/37 17:29/49 24:29/50 32:32/52 33:47/62 48:54/65 64:58/78
 """
 
 
